@@ -373,222 +373,157 @@ __global__ void __launch_bounds__(kSlotThreads)
         if (e[i] < elems) store_sem<VEC>(sem + slot * elems + e[i], v[i]);
 }
 
-// The per-slot fold with the states streamed through shared memory by the TMA
-// engine. A persistent CTA takes a contiguous run of (slot, element range)
-// tiles. Its producer warp streams the slot ids through a ring of kIdRing
-// chunks of kIdChunk ids (bulk copies kIdRing chunks ahead, so that finding
-// the deposits does not wait on one round trip per chunk), matches them in
-// deposit order and, for each deposit of the tile's slot, queues one bulk copy
-// of that deposit's range of elements into a ring of kRing stages; the
-// kBulkConsumers consumer threads fold every stage into the range's semantic
-// values, which stay in registers for the whole tile. A stage tagged
-// kTagTileEnd carries no data and closes the tile: its values are stored and
-// the next tile's loaded while the ring keeps streaming. Each state element
-// crosses HBM once, each semantic element is read and written once.
-constexpr int kBulkConsumers = 256;
-constexpr int kBulkThreads = kBulkConsumers + 32;
-constexpr int kStageBytes = 16384;
-constexpr int kRing = 6;
-constexpr int kChunksPerThread = kStageBytes / 16 / kBulkConsumers;
-constexpr int kIdChunk = 256;
-constexpr int kIdRing = 6;
-constexpr int32_t kTagData = 1;
-constexpr int32_t kTagTileEnd = 2;
-static_assert(kChunksPerThread * 16 * kBulkConsumers == kStageBytes, "stage = whole 16-byte chunks");
-static_assert(kIdChunk % 32 == 0, "whole warps of ids");
+// The per-slot fold with the states streamed through shared memory by asynchronous
+// copies. HBM-bound: each state element crosses HBM once and each touched semantic
+// element is read and written once; slots without a deposit are not read.
+//
+// Split: deposits are spread unevenly over slots (a slot may hold a fifth of them),
+// and one element's deposits form a serial chain, so the work is divided by bytes,
+// not by slots. Every CTA counts the deposits of each slot, weighs a slot's unit of
+// kUnitBytes by the bytes it moves, and takes an equal share of the total weight: a
+// contiguous run of (slot, element range) pieces, ranges of any width. Fixed 16 KB
+// ranges in contiguous runs instead left 240 CTAs waiting for the few that held the
+// largest slot.
+//
+// A piece is processed in tiles of at most kTileBytes. The CTA lists the slot's
+// deposits in deposit order (ballots over the slot ids, kWindow at a time) and every
+// thread then folds its own 16-byte chunks of the tile, in deposit order, through a
+// private ring of 16-byte asynchronous copies in shared memory: no barrier, no producer
+// and no wait on another thread. (One producer thread queueing a bulk copy per deposit
+// cost about 250 ns per deposit and CTA, whatever the size: 1.0 TB/s on 2 KB ranges.)
+// kRingChunks chunks per thread are in flight: 18 deposits of a tile of up to 4 KB, 9 of
+// 8 KB, 4 of 16 KB, 3 of 24 KB, 72 KB per CTA and two CTAs per SM. Narrower or wider tiles
+// and shorter or longer rings were slower (4096 states below: 16 KB tiles 147 us; a ring of
+// 12 chunks 158 us; 24 chunks the same as 18 and 66 against 64 us in the second case).
+//
+// 24-layer bf16 states (192 KB each), before -> now:
+//   4096 into 64 slots, evenly                     137.6 -> 137.9 us  (6.21 TB/s)
+//   1500 into 80 slots, evenly                      69.6 ->  63.9 us
+//   1500 into 80 slots, 40 % of them in 4 slots    247   ->  66.2 us
+//   1073 into 3 slots                              132   ->  82.9 us
+//   4096 into 1 slot                              4202   -> 437   us
+constexpr int kFoldThreads = 256;
+constexpr int kFoldWarps = kFoldThreads / 32;
+constexpr int kRingChunks = 18;    // 16-byte chunks in flight per thread
+constexpr int kTileChunks = 6;     // 16-byte chunks of a tile per thread, at most
+constexpr int kTileBytes = kTileChunks * 16 * kFoldThreads;
+constexpr int kUnitBytes = 512;    // granularity of a piece
+constexpr int kTallySlots = kFoldThreads;   // slots counted in shared memory, one per thread
+constexpr int kIdsPerLane = 16;
+constexpr int kWindow = kFoldThreads * kIdsPerLane;   // slot ids listed at once
+static_assert(kWindow <= 65536, "list entries are 16-bit");
 
-struct BulkSmem {
-    unsigned char ring[kRing][kStageBytes];
-    int64_t ids[kIdRing][kIdChunk];
-    uint64_t full[kRing];
-    uint64_t empty[kRing];
-    uint64_t idfull[kIdRing];
-    int32_t tag[kRing];
-    int32_t abort;
+struct FoldSmem {
+    uint4 ring[kRingChunks * kFoldThreads];
+    uint16_t list[kWindow];         // positions in the window of the slot's deposits
+    int64_t wsum[kFoldWarps];       // sums of 32 slots' weights
+    int32_t count[kTallySlots];     // deposits per slot
+    int32_t begin[kTallySlots];     // this CTA's units of each slot: [begin, end)
+    int32_t end[kTallySlots];
+    int32_t warp_hits[kFoldWarps];
+    int32_t first_slot, last_slot;  // slots with a piece of this CTA
 };
 
-// Bounded wait that also gives up once another role of the CTA has given up.
-__device__ __forceinline__ bool wait_or_abort(uint64_t *bar, uint32_t parity, const volatile int32_t *abort) {
-    for (uint32_t i = 0; i < kWaitLimit; ++i) {
-        if (mbar_try_wait(bar, parity)) return true;
-        if ((i & 255u) == 255u && *abort) return false;
-    }
-    return false;
+// Tiles of a piece of `len` units: as few as fit, of equal width (in units).
+__device__ __forceinline__ int tile_units(int len) {
+    constexpr int kMost = kTileBytes / kUnitBytes;
+    const int tiles = (len + kMost - 1) / kMost;
+    return (len + tiles - 1) / tiles;
 }
 
-// Producer: claim stage g (wait until the consumers released its previous
-// use), tag it and start its copy (src == nullptr: a tile-end marker).
-// Warp-uniform result; false when the wait ran out or the CTA gave up.
-__device__ __forceinline__ bool produce_stage(BulkSmem &sm, uint32_t g, int lane, const void *src,
-                                              uint32_t bytes) {
-    const int s = static_cast<int>(g % kRing);
-    int ok = 1;
-    if (lane == 0) {
-        ok = wait_or_abort(&sm.empty[s], ((g / kRing) & 1u) ^ 1u, &sm.abort);
-        if (ok) {
-            sm.tag[s] = src ? kTagData : kTagTileEnd;
-            if (src) {
-                mbar_arrive_expect_tx(&sm.full[s], bytes);
-                bulk_g2s(sm.ring[s], src, bytes, &sm.full[s]);
-            } else {
-                mbar_arrive(&sm.full[s]);
-            }
-        }
+// Lists the deposits of `slot` among ids [c0, c0 + kWindow) in order; their number.
+// Every thread of the block; the previous list may still be read until it starts.
+__device__ __forceinline__ int list_deposits(FoldSmem &sm, const int64_t *__restrict__ slots, int64_t n, int64_t c0,
+                                             int slot) {
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    uint32_t hits[kIdsPerLane];
+    int64_t id[kIdsPerLane];
+#pragma unroll
+    for (int r = 0; r < kIdsPerLane; ++r) {
+        const int64_t c = c0 + (warp * kIdsPerLane + r) * 32 + lane;
+        id[r] = c < n ? slots[c] : -1;
     }
-    return __shfl_sync(0xffffffffu, ok, 0) != 0;
-}
-
-// Producer lane 0: start id chunk k of the scan (ids [k * kIdChunk, ...)), the u-th
-// chunk of the CTA, into id stage u % kIdRing. An odd count leaves its last id to a
-// plain load (bulk sizes are multiples of 16).
-__device__ __forceinline__ void issue_ids(BulkSmem &sm, const int64_t *__restrict__ slots, int64_t n, int64_t k,
-                                          int64_t u) {
-    const int s = static_cast<int>(u % kIdRing);
-    const int64_t c0 = k * kIdChunk;
-    const int64_t cnt = n - c0 < kIdChunk ? n - c0 : kIdChunk;
-    const uint32_t bytes = static_cast<uint32_t>((cnt & ~static_cast<int64_t>(1)) * 8);
-    if (bytes == 0) {
-        mbar_arrive(&sm.idfull[s]);
-    } else {
-        mbar_arrive_expect_tx(&sm.idfull[s], bytes);
-        bulk_g2s(sm.ids[s], slots + c0, bytes, &sm.idfull[s]);
-    }
-}
-
-template <typename TS>
-__global__ void __launch_bounds__(kBulkThreads, 2)
-    smc_consolidate_bulk_kernel(float *__restrict__ sem, int64_t n_slots, int64_t elems,
-                                const TS *__restrict__ states, const int64_t *__restrict__ slots,
-                                int64_t n, float alpha, int64_t ntiles, int64_t per_cta) {
-    constexpr int CH = 16 / static_cast<int>(sizeof(TS));          // state elements per 16-byte chunk
-    constexpr int64_t R = kStageBytes / static_cast<int64_t>(sizeof(TS));  // elements per tile
-    extern __shared__ __align__(16) unsigned char smem_raw[];
-    BulkSmem &sm = *reinterpret_cast<BulkSmem *>(smem_raw);
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    const int64_t nranges = (elems + R - 1) / R;
-    const int64_t t_begin = static_cast<int64_t>(blockIdx.x) * per_cta;
-    const int64_t t_end = t_begin + per_cta < ntiles ? t_begin + per_cta : ntiles;
-    if (tid == 0) {
-        for (int s = 0; s < kRing; ++s) {
-            mbar_init(&sm.full[s], 1);
-            mbar_init(&sm.empty[s], kBulkConsumers / 32);
-        }
-        for (int s = 0; s < kIdRing; ++s) mbar_init(&sm.idfull[s], 1);
-        sm.abort = 0;
-        fence_barrier_init();
+    int mine = 0;
+#pragma unroll
+    for (int r = 0; r < kIdsPerLane; ++r) {
+        hits[r] = __ballot_sync(0xffffffffu, id[r] == slot);
+        mine += __popc(hits[r]);
     }
     __syncthreads();
-
-    if (warp == kBulkConsumers / 32) {
-        // ---- producer warp ----
-        uint32_t g = 0;        // ring stages produced
-        int64_t kid = 0;       // id chunks consumed (all tiles)
-        int64_t kid_issued = 0;
-        bool ok = true;
-        const int64_t nchunks = (n + kIdChunk - 1) / kIdChunk;
-        for (int64_t t = t_begin; t < t_end && ok; ++t) {
-            const int64_t slot = t / nranges;
-            const int64_t e0 = (t % nranges) * R;
-            const int64_t rlen = elems - e0 < R ? elems - e0 : R;
-            const uint32_t bytes = static_cast<uint32_t>(rlen * static_cast<int64_t>(sizeof(TS)));
-            const TS *src = states + e0;
-            const bool flagger = t == 0;
-            const int64_t base = kid;
-            const int64_t first = nchunks < kIdRing ? nchunks : kIdRing;
-            if (lane == 0) {
-                fence_proxy_async_smem();   // the previous tile's reads of the id stages precede their refill
-                for (int64_t k = 0; k < first; ++k) issue_ids(sm, slots, n, k, base + k);
-            }
-            kid_issued = base + first;
-            for (int64_t k = 0; k < nchunks && ok; ++k, ++kid) {
-                const int is = static_cast<int>(kid % kIdRing);
-                int waited = 1;
-                if (lane == 0) waited = wait_or_abort(&sm.idfull[is], static_cast<uint32_t>((kid / kIdRing) & 1), &sm.abort);
-                if (__shfl_sync(0xffffffffu, waited, 0) == 0) {
-                    ok = false;
-                    break;
-                }
-                const int64_t c0 = k * kIdChunk;
-                const int64_t cnt = n - c0 < kIdChunk ? n - c0 : kIdChunk;
-                const int64_t cnt_even = cnt & ~static_cast<int64_t>(1);
+    if (lane == 0) sm.warp_hits[warp] = mine;
+    __syncthreads();
+    int at = 0, total = 0;
 #pragma unroll
-                for (int p = 0; p < kIdChunk / 32; ++p) {
-                    const int j = p * 32 + lane;
-                    const int64_t id = j < cnt_even ? sm.ids[is][j] : (j < cnt ? slots[c0 + j] : -1);
-                    if (flagger && (id >= n_slots || id < -1)) atomicOr(&g_smc_status, PRECOG_DEV_BAD_INDEX);
-                    uint32_t ball = __ballot_sync(0xffffffffu, id == slot);
-                    while (ball != 0u && ok) {
-                        const int jj = __ffs(static_cast<int>(ball)) - 1;
-                        ball &= ball - 1u;
-                        ok = produce_stage(sm, g, lane, src + (c0 + p * 32 + jj) * elems, bytes);
-                        if (ok) ++g;
-                    }
-                }
-                __syncwarp();
-                if (ok && k + kIdRing < nchunks) {
-                    if (lane == 0) {
-                        fence_proxy_async_smem();   // the warp's reads of this id stage precede its refill
-                        issue_ids(sm, slots, n, k + kIdRing, base + k + kIdRing);
-                    }
-                    ++kid_issued;
-                }
-            }
-            if (ok) {
-                ok = produce_stage(sm, g, lane, nullptr, 0);
-                if (ok) ++g;
-            }
-        }
-        if (!ok && lane == 0) {
-            // Give up: record it, stop the consumers, let the issued copies land.
-            atomicOr(&g_smc_status, PRECOG_DEV_TIMEOUT);
-            *static_cast<volatile int32_t *>(&sm.abort) = 1;
-            for (uint32_t g2 = g > kRing ? g - kRing : 0; g2 < g; ++g2)
-                mbar_wait(&sm.full[g2 % kRing], (g2 / kRing) & 1u);
-            for (int64_t u = kid; u < kid_issued; ++u)
-                mbar_wait(&sm.idfull[u % kIdRing], static_cast<uint32_t>((u / kIdRing) & 1));
-        }
-        return;
+    for (int w = 0; w < kFoldWarps; ++w) {
+        const int h = sm.warp_hits[w];
+        at += w < warp ? h : 0;
+        total += h;
     }
+#pragma unroll
+    for (int r = 0; r < kIdsPerLane; ++r) {
+        if (hits[r] >> lane & 1u)
+            sm.list[at + __popc(hits[r] & ((1u << lane) - 1u))] = static_cast<uint16_t>((warp * kIdsPerLane + r) * 32 + lane);
+        at += __popc(hits[r]);
+    }
+    __syncthreads();
+    return total;
+}
 
-    // ---- consumer warps ----
+// One tile of `rlen` elements of `slot`'s row (`srow`, and `src` in the deposits' rows), C
+// 16-byte chunks for each of kFoldThreads / B threads. The other threads' ring slots hold
+// B deposits side by side. listed >= 0: the list already holds all deposits of the slot.
+template <typename TS, int C, int B>
+__device__ __forceinline__ void fold_tile(FoldSmem &sm, float *__restrict__ srow, const TS *__restrict__ src,
+                                          int64_t rlen, int64_t elems, const int64_t *__restrict__ slots, int64_t n,
+                                          int slot, int listed, float alpha) {
+    constexpr int CH = 16 / static_cast<int>(sizeof(TS));   // state elements per chunk
+    constexpr int P = kRingChunks / C;                      // groups of B deposits in the ring
+    constexpr int W = kFoldThreads / B;                     // threads with chunks
+    static_assert(B == 1 || C == 1, "side by side only in narrow tiles");
+    const int tid = threadIdx.x;
     const float keep = 1.f - alpha;
-    uint32_t g = 0;
-    for (int64_t t = t_begin; t < t_end; ++t) {
-        const int64_t slot = t / nranges;
-        const int64_t e0 = (t % nranges) * R;
-        const int64_t rlen = elems - e0 < R ? elems - e0 : R;
-        float *srow = sem + slot * elems + e0;
-        float v[kChunksPerThread][CH];
-        bool have[kChunksPerThread];
+    float v[C][CH];
+    bool have[C];
 #pragma unroll
-        for (int i = 0; i < kChunksPerThread; ++i) {
-            const int64_t q = static_cast<int64_t>(i) * kBulkConsumers + tid;
-            have[i] = q * CH < rlen;
+    for (int i = 0; i < C; ++i) {
+        const int64_t q = static_cast<int64_t>(i * kFoldThreads + tid) * CH;
+        have[i] = q < rlen && tid < W;
 #pragma unroll
-            for (int k = 0; k < CH; k += 4) {
-                float4 f = make_float4(0.f, 0.f, 0.f, 0.f);
-                if (have[i]) f = *reinterpret_cast<const float4 *>(srow + q * CH + k);
-                v[i][k] = f.x;
-                v[i][k + 1] = f.y;
-                v[i][k + 2] = f.z;
-                v[i][k + 3] = f.w;
-            }
+        for (int k = 0; k < CH; k += 4) {
+            const float4 f = have[i] ? *reinterpret_cast<const float4 *>(srow + q + k) : make_float4(0.f, 0.f, 0.f, 0.f);
+            v[i][k] = f.x;
+            v[i][k + 1] = f.y;
+            v[i][k + 2] = f.z;
+            v[i][k + 3] = f.w;
         }
-        bool touched = false;
-        while (true) {
-            const int s = static_cast<int>(g % kRing);
-            if (!wait_or_abort(&sm.full[s], (g / kRing) & 1u, &sm.abort)) {
-                if (lane == 0) atomicOr(&g_smc_status, PRECOG_DEV_TIMEOUT);
-                *static_cast<volatile int32_t *>(&sm.abort) = 1;
-                return;
-            }
-            const int32_t tag = sm.tag[s];
-            if (tag == kTagData) {
+    }
+    for (int64_t c0 = 0; c0 < n; c0 += kWindow) {
+        const int m = listed >= 0 ? listed : list_deposits(sm, slots, n, c0, slot);
+        const TS *base = src + c0 * elems + static_cast<int64_t>(tid) * CH;
+        int in = 0, out = 0;   // ring positions of the next group copied and folded
+        auto copy = [&](int j0) {
 #pragma unroll
-                for (int i = 0; i < kChunksPerThread; ++i) {
+            for (int b = 0; b < B; ++b)
+                if (j0 + b < m) {
+                    const TS *row = base + static_cast<int64_t>(sm.list[j0 + b]) * elems;
+#pragma unroll
+                    for (int i = 0; i < C; ++i)
+                        if (have[i])
+                            cp_async16(&sm.ring[(in * C + i) * kFoldThreads + b * W + tid], row + i * kFoldThreads * CH);
+                }
+            cp_async_commit();
+            in = in + 1 == P ? 0 : in + 1;
+        };
+        for (int j = 0; j < (P - 1) * B; j += B) copy(j);
+        for (int j = 0; j < m; j += B) {
+            cp_async_wait<P - 2>();
+#pragma unroll
+            for (int b = 0; b < B; ++b) {
+                if (j + b >= m) break;
+#pragma unroll
+                for (int i = 0; i < C; ++i) {
                     if (!have[i]) continue;
-                    const uint4 raw = *reinterpret_cast<const uint4 *>(
-                        sm.ring[s] + (static_cast<int>(i) * kBulkConsumers + tid) * 16);
+                    const uint4 raw = sm.ring[(out * C + i) * kFoldThreads + b * W + tid];
                     float h[CH];
                     if constexpr (std::is_same<TS, float>::value) {
                         h[0] = __uint_as_float(raw.x);
@@ -606,23 +541,113 @@ __global__ void __launch_bounds__(kBulkThreads, 2)
 #pragma unroll
                     for (int k = 0; k < CH; ++k) v[i][k] = fmaf(keep, v[i][k], alpha * h[k]);
                 }
-                touched = true;
             }
-            __syncwarp();
-            if (lane == 0) mbar_arrive(&sm.empty[s]);
-            ++g;
-            if (tag != kTagData) break;
+            out = out + 1 == P ? 0 : out + 1;
+            copy(j + (P - 1) * B);
         }
-        if (touched) {
+        cp_async_wait<0>();
+    }
 #pragma unroll
-            for (int i = 0; i < kChunksPerThread; ++i) {
-                if (!have[i]) continue;
-                const int64_t q = static_cast<int64_t>(i) * kBulkConsumers + tid;
+    for (int i = 0; i < C; ++i) {
+        if (!have[i]) continue;
+        const int64_t q = static_cast<int64_t>(i * kFoldThreads + tid) * CH;
 #pragma unroll
-                for (int k = 0; k < CH; k += 4)
-                    *reinterpret_cast<float4 *>(srow + q * CH + k) =
-                        make_float4(v[i][k], v[i][k + 1], v[i][k + 2], v[i][k + 3]);
-            }
+        for (int k = 0; k < CH; k += 4)
+            *reinterpret_cast<float4 *>(srow + q + k) = make_float4(v[i][k], v[i][k + 1], v[i][k + 2], v[i][k + 3]);
+    }
+}
+
+template <typename TS>
+__global__ void __launch_bounds__(kFoldThreads, 2)
+    smc_consolidate_share_kernel(float *__restrict__ sem, int n_slots, int64_t elems, const TS *__restrict__ states,
+                                 const int64_t *__restrict__ slots, int64_t n, float alpha) {
+    constexpr int64_t U = kUnitBytes / static_cast<int64_t>(sizeof(TS));  // elements per unit
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    FoldSmem &sm = *reinterpret_cast<FoldSmem *>(smem_raw);
+    const int tid = threadIdx.x;
+    const int64_t units = (elems + U - 1) / U;
+    if (tid == 0) {
+        sm.first_slot = n_slots;
+        sm.last_slot = -1;
+    }
+    sm.count[tid] = 0;
+    __syncthreads();
+
+    // ---- this CTA's pieces ----
+    constexpr int kAhead = 16;   // slot ids in flight per thread
+    for (int64_t c0 = 0; c0 < n; c0 += kAhead * kFoldThreads) {
+        int64_t id[kAhead];
+#pragma unroll
+        for (int r = 0; r < kAhead; ++r) {
+            const int64_t c = c0 + r * kFoldThreads + tid;
+            id[r] = c < n ? slots[c] : -1;
+        }
+#pragma unroll
+        for (int r = 0; r < kAhead; ++r) {
+            if (id[r] >= 0 && id[r] < n_slots) atomicAdd(&sm.count[id[r]], 1);
+            else if (id[r] != -1 && blockIdx.x == 0) atomicOr(&g_smc_status, PRECOG_DEV_BAD_INDEX);
+        }
+    }
+    __syncthreads();
+    // a unit of a touched slot moves count * kUnitBytes of states and its semantic values
+    // twice (8 bytes an element); weights in units of kUnitBytes, thread s sums slots 0..s
+    constexpr int64_t kSemWeight = 2 * U * 4 / kUnitBytes;
+    const int64_t w = sm.count[tid] > 0 ? sm.count[tid] + kSemWeight : 0;
+    int64_t upto = w;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const int64_t v = __shfl_up_sync(0xffffffffu, upto, o);
+        upto += (tid & 31) >= o ? v : 0;
+    }
+    if ((tid & 31) == 31) sm.wsum[tid >> 5] = upto;
+    __syncthreads();
+    int64_t total = 0;
+#pragma unroll
+    for (int v = 0; v < kFoldWarps; ++v) {
+        const int64_t t = sm.wsum[v];
+        upto += v < (tid >> 5) ? t : 0;
+        total += t;
+    }
+    total *= units;
+    if (w > 0) {
+        // unit u of slot s covers weights [base + u * w, base + (u + 1) * w); this CTA
+        // takes the units that start in [lo, hi)
+        const int64_t share = total / gridDim.x, rest = total % gridDim.x;
+        const int64_t b = blockIdx.x;
+        const int64_t lo = b * share + (b < rest ? b : rest);
+        const int64_t hi = lo + share + (b < rest ? 1 : 0);
+        const int64_t base = (upto - w) * units;
+        const int64_t u0 = lo > base ? (lo - base + w - 1) / w : 0;
+        const int64_t u1 = hi > base ? (hi - base + w - 1) / w : 0;
+        sm.begin[tid] = static_cast<int32_t>(u0 < units ? u0 : units);
+        sm.end[tid] = static_cast<int32_t>(u1 < units ? u1 : units);
+        if (sm.begin[tid] < sm.end[tid]) {
+            atomicMin(&sm.first_slot, tid);
+            atomicMax(&sm.last_slot, tid);
+        }
+    }
+    __syncthreads();
+
+    const int last_slot = sm.last_slot;
+    for (int slot = sm.first_slot; slot <= last_slot; ++slot) {
+        if (sm.count[slot] == 0) continue;
+        const int begin = sm.begin[slot], end = sm.end[slot];
+        if (begin >= end) continue;
+        const int listed = n <= kWindow ? list_deposits(sm, slots, n, 0, slot) : -1;
+        const int step = tile_units(end - begin);
+        const int chunks = step * (kUnitBytes / 16);
+        for (int u = begin; u < end; u += step) {
+            const int64_t e0 = u * U;
+            const int64_t e1 = (u + step < end ? u + step : end) * U;
+            const int64_t rlen = (e1 < elems ? e1 : elems) - e0;
+            float *srow = sem + static_cast<int64_t>(slot) * elems + e0;
+            const TS *src = states + e0;
+            if (chunks * 4 <= kFoldThreads) fold_tile<TS, 1, 4>(sm, srow, src, rlen, elems, slots, n, slot, listed, alpha);
+            else if (chunks * 2 <= kFoldThreads) fold_tile<TS, 1, 2>(sm, srow, src, rlen, elems, slots, n, slot, listed, alpha);
+            else if (chunks <= kFoldThreads) fold_tile<TS, 1, 1>(sm, srow, src, rlen, elems, slots, n, slot, listed, alpha);
+            else if (chunks <= 2 * kFoldThreads) fold_tile<TS, 2, 1>(sm, srow, src, rlen, elems, slots, n, slot, listed, alpha);
+            else if (chunks <= 4 * kFoldThreads) fold_tile<TS, 4, 1>(sm, srow, src, rlen, elems, slots, n, slot, listed, alpha);
+            else fold_tile<TS, kTileChunks, 1>(sm, srow, src, rlen, elems, slots, n, slot, listed, alpha);
         }
     }
 }
@@ -677,30 +702,29 @@ cudaError_t launch_smc_consolidate(float *sem, int64_t n_slots, int64_t elems, c
     const int64_t blocks = (elems / vec + kConsThreads - 1) / kConsThreads;
     if (blocks > 0x7fffffffLL) return cudaErrorInvalidConfiguration;
     const unsigned grid = static_cast<unsigned>(blocks);
-    // Few slots: CTAs per (slot, element range). Each tile reads all n slot ids (from
-    // L2): n_slots / 2048 of its state bytes with 16 KB ranges, so it pays up to 256
-    // slots. Rows of whole 16-byte chunks stream through the TMA ring; other rows take
-    // the register per-slot kernel (whose 2048-element ranges read n_slots / 512).
-    const int64_t chunk = states_dtype == PRECOG_BF16 ? 8 : 4;
-    if (n_slots >= 1 && n_slots <= 256 && elems % chunk == 0 && reinterpret_cast<uintptr_t>(slots) % 16 == 0) {
-        const int64_t range = kStageBytes / (states_dtype == PRECOG_BF16 ? 2 : 4);
-        const int64_t ntiles = n_slots * ((elems + range - 1) / range);
+    // Few slots: CTAs over pieces of (slot, element range). Each piece (each tile beyond
+    // kWindow deposits) reads all n slot ids from L2: n_slots / 2048 of its state bytes
+    // with 16 KB ranges, so it pays up to 256 slots. Rows of whole 16-byte chunks stream
+    // through the copy ring; other rows take the register per-slot kernel (whose
+    // 2048-element ranges read n_slots / 512).
+    const int64_t size = states_dtype == PRECOG_BF16 ? 2 : 4;
+    const int64_t units = (elems * size + kUnitBytes - 1) / kUnitBytes;
+    if (n_slots >= 1 && n_slots <= kTallySlots && elems * size % 16 == 0 && units < 0x7fffffffLL) {
         const int64_t resident = 2 * static_cast<int64_t>(device_sm_count());
-        const int64_t per_cta = (ntiles + resident - 1) / resident;
-        const int64_t blocks2 = (ntiles + per_cta - 1) / per_cta;
-        if (blocks2 > 0x7fffffffLL) return cudaErrorInvalidConfiguration;
-        const int smem = static_cast<int>(sizeof(BulkSmem));
+        const int64_t touched = n < n_slots ? n : n_slots;   // at most
+        const int64_t blocks2 = touched * units < resident ? touched * units : resident;
+        const int smem = static_cast<int>(sizeof(FoldSmem));
         cudaError_t e;
         if (states_dtype == PRECOG_BF16) {
-            e = ensure_smem(reinterpret_cast<const void *>(smc_consolidate_bulk_kernel<__nv_bfloat16>), smem);
+            e = ensure_smem(reinterpret_cast<const void *>(smc_consolidate_share_kernel<__nv_bfloat16>), smem);
             if (e != cudaSuccess) return e;
-            smc_consolidate_bulk_kernel<__nv_bfloat16><<<static_cast<unsigned>(blocks2), kBulkThreads, smem, stream>>>(
-                sem, n_slots, elems, static_cast<const __nv_bfloat16 *>(states), slots, n, alpha, ntiles, per_cta);
+            smc_consolidate_share_kernel<__nv_bfloat16><<<static_cast<unsigned>(blocks2), kFoldThreads, smem, stream>>>(
+                sem, static_cast<int>(n_slots), elems, static_cast<const __nv_bfloat16 *>(states), slots, n, alpha);
         } else {
-            e = ensure_smem(reinterpret_cast<const void *>(smc_consolidate_bulk_kernel<float>), smem);
+            e = ensure_smem(reinterpret_cast<const void *>(smc_consolidate_share_kernel<float>), smem);
             if (e != cudaSuccess) return e;
-            smc_consolidate_bulk_kernel<float><<<static_cast<unsigned>(blocks2), kBulkThreads, smem, stream>>>(
-                sem, n_slots, elems, static_cast<const float *>(states), slots, n, alpha, ntiles, per_cta);
+            smc_consolidate_share_kernel<float><<<static_cast<unsigned>(blocks2), kFoldThreads, smem, stream>>>(
+                sem, static_cast<int>(n_slots), elems, static_cast<const float *>(states), slots, n, alpha);
         }
         e = cudaGetLastError();
         if (e == cudaSuccess) count_launches(1);

@@ -233,3 +233,33 @@ def test_smc_benchmark_sizes_sampled(cuda_device):
     got = to_np(sem[:, cols])
     for s in range(64):
         assert rel_err(got[s], ref[s]) < TOL_F32, s
+
+
+@pytest.mark.parametrize("dtype,elems,n,n_slots,heavy", [
+    ("bf16", 98304, 60, 16, 0.5), ("bf16", 264, 5, 256, 0.2), ("f32", 20004, 333, 3, 0.9),
+    ("f32", 124, 700, 2, 0.99), ("bf16", 8200, 300, 255, 0.0), ("bf16", 16384 * 3, 9, 9, 0.0)])
+def test_consolidate_uneven_slots(cuda_device, dtype, elems, n, n_slots, heavy):
+    """The staged fold divides the bytes of unevenly filled slots evenly over its CTAs: one
+    slot with a share `heavy` of the deposits, slots without any (left bit for bit), pieces
+    narrower and wider than a stage, rows that end inside a unit. Every element takes its
+    deposits in order (each fp32 step rounds within 2^-23 of its operands)."""
+    import torch
+    import paper_2608_02560_gb300 as pg
+    rng = np.random.default_rng(elems + n)
+    states = torch.from_numpy(rng.standard_normal((n, elems)).astype(np.float32)).to(cuda_device)
+    if dtype == "bf16":
+        states = states.to(torch.bfloat16)
+    slot_np = rng.integers(0, n_slots, size=n).astype(np.int64)
+    slot_np[rng.random(n) < heavy] = n_slots // 2
+    slot_np[rng.random(n) < 0.1] = -1
+    sem0 = rng.standard_normal((n_slots, elems)).astype(np.float32)
+    sem = torch.from_numpy(sem0).to(cuda_device)
+    pg.precog_smc_consolidate(sem, states, torch.from_numpy(slot_np).to(cuda_device), 0.3)
+    assert pg.precog_device_status()[0] == 0
+    ref = oracle.smc_consolidate(sem0, to_np(states.float()), slot_np, 0.3)
+    got = to_np(sem)
+    for s in range(n_slots):
+        if s in slot_np:
+            assert rel_err(got[s], ref[s]) < TOL_F32, s
+        else:
+            np.testing.assert_array_equal(got[s], sem0[s])
