@@ -1,6 +1,8 @@
 // Exact top-1 dot-product retrieval over a flat key index (Sec. 4.2).
 //
-// Batched GEMV on the CUDA cores: every warp streams whole key rows with
+// fp32 keys, on the CUDA cores (16-bit keys: retrieve_tc.cu). Batches share each row among
+// the warps of a CTA (gemm_retrieve_kernel below). The GEMV kernels take a single query's short
+// rows and the longest rows: every warp streams whole key rows with
 // 16-byte loads (several rows in flight per warp), dots them with a group of
 // up to kQB queries held in registers as fp32, and reduces across lanes with
 // a fixed butterfly, so a row's score never depends on where the row sits:
@@ -153,7 +155,7 @@ __device__ __forceinline__ int64_t global_key(unsigned long long k, int64_t row_
     return static_cast<int64_t>(k ^ 0x8000000000000000ull);
 }
 
-__device__ __forceinline__ void write_best(unsigned long long k, int64_t *best_idx, float *best_score, int q) {
+__device__ __forceinline__ void write_best(unsigned long long k, int64_t *best_idx, float *best_score, int64_t q) {
     if (k == 0ull) {
         best_idx[q] = -1;
         if (best_score) best_score[q] = __uint_as_float(0x7fc00000u);
@@ -291,43 +293,302 @@ __global__ void __launch_bounds__(kThreads)
     }
 }
 
-// Merge the per-CTA lists of one query into its k best, one warp per query:
-// each lane merges a strided share of the CTAs' lists, then five butterfly
-// rounds merge the lanes' lists (keys are unique, so both partners of a round
-// end with the same list).
-__global__ void finalize_topk_kernel(const unsigned long long *__restrict__ partial, int n_parts,
+__device__ __forceinline__ unsigned long long warp_max_u64(unsigned long long v) {
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+        const unsigned long long w = shfl_xor_u64(v, o);
+        v = w > v ? w : v;
+    }
+    return v;
+}
+
+// Merge the per-CTA lists of one query into its k best, one warp per query. The lists'
+// 2^log_used leading entries (of kListK) are spread over the lanes, kAhead independent
+// loads at a time. The k-th largest of the lanes' largest heads bounds the k-th best from
+// below, so few entries reach a lane's sorted list; then k rounds take the warp's largest
+// head (keys are unique, so one lane owns it and drops it). One list per lane with
+// dependent loads, merged by butterflies, took 25 us for 608 parts.
+__global__ void finalize_topk_kernel(const unsigned long long *__restrict__ partial, int n_parts, int log_used,
                                      int n_queries, int k, int64_t *__restrict__ best_idx,
                                      float *__restrict__ best_score) {
+    constexpr int kAhead = 8;
     const int q = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const int lane = threadIdx.x & 31;
     if (q >= n_queries) return;
+    auto entry = [&](int part, int j) {
+        return partial[(static_cast<int64_t>(part) * n_queries + q) * kListK + j];
+    };
+    unsigned long long head = 0ull;
+    for (int i0 = lane; i0 < n_parts; i0 += 32 * kAhead) {
+        unsigned long long v[kAhead];
+#pragma unroll
+        for (int r = 0; r < kAhead; ++r) v[r] = i0 + 32 * r < n_parts ? entry(i0 + 32 * r, 0) : 0ull;
+#pragma unroll
+        for (int r = 0; r < kAhead; ++r) head = v[r] > head ? v[r] : head;
+    }
+    unsigned long long least = 0ull;
+    for (int j = 0; j < k; ++j) {
+        least = warp_max_u64(head);
+        if (head == least) head = 0ull;
+    }
     unsigned long long l[kListK];
 #pragma unroll
     for (int j = 0; j < kListK; ++j) l[j] = 0ull;
-    for (int i = lane; i < n_parts; i += 32)
-        for (int j = 0; j < kListK; ++j) {
-            const unsigned long long v = partial[(static_cast<int64_t>(i) * n_queries + q) * kListK + j];
-            if (v <= l[kListK - 1]) break;   // each part's list is sorted: the rest is smaller
-            list_insert(l, v);
+    const int total = n_parts << log_used, mask = (1 << log_used) - 1;
+    for (int i0 = lane; i0 < total; i0 += 32 * kAhead) {
+        unsigned long long v[kAhead];
+#pragma unroll
+        for (int r = 0; r < kAhead; ++r) {
+            const int i = i0 + 32 * r;
+            v[r] = i < total ? entry(i >> log_used, i & mask) : 0ull;
         }
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-        unsigned long long other[kListK];
-#pragma unroll
-        for (int j = 0; j < kListK; ++j) other[j] = shfl_xor_u64(l[j], o);
-#pragma unroll
-        for (int j = 0; j < kListK; ++j) list_insert(l, other[j]);
+        for (int r = 0; r < kAhead; ++r)
+            if (v[r] >= least) list_insert(l, v[r]);
     }
-    if (lane != 0) return;
     for (int j = 0; j < k; ++j) {
-        const unsigned long long key = l[j];
-        const int64_t o = static_cast<int64_t>(q) * k + j;
-        if (key == 0ull) {
-            best_idx[o] = -1;
-            if (best_score) best_score[o] = __uint_as_float(0x7fc00000u);
+        const unsigned long long key = warp_max_u64(l[0]);
+        if (key != 0ull && key == l[0]) {
+#pragma unroll
+            for (int i = 0; i + 1 < kListK; ++i) l[i] = l[i + 1];
+            l[kListK - 1] = 0ull;
+        }
+        if (lane == 0) write_best(key, best_idx, best_score, static_cast<int64_t>(q) * k + j);
+    }
+}
+
+// ---------------------------------------------------------------------------
+// Batches over an fp32 index: one pass over the keys for up to kGemmWarps * QW queries.
+//
+// fp32 scores stay on the FMA pipe (the tensor cores would round the keys). A pass per 4
+// queries (top-1) or per query (top-k) re-read the index once per pass; here a CTA streams
+// tiles of whole key rows through a shared-memory ring (one bulk copy per tile, the rows
+// being contiguous) and its kGemmWarps warps share them: WQ groups of QW queries times WR
+// shares of the tile's row pairs. A lane owns the 16-byte vectors l, l+32, ... of a row, as
+// in the GEMV, with its QW queries' values in registers, so a row costs VPL 16-byte
+// shared-memory reads per QW * VPL * 4 multiply-adds (packed, adjacent dims in the halves);
+// with QW = 8 shared memory is half as busy as the FMA pipe, with QW = 4 (rows over 384
+// dims: the query registers) as busy. The 2 * QW sums of a row pair are added across the
+// lanes by halving exchanges (each step sends the half of the sums that the other lane
+// keeps): 16 exchanges for 16 sums where separate butterflies take 80, in the same tree for
+// every row, so equal rows score equally. Bound: HBM up to about 8 queries, then the FMA
+// pipe (56 % busy: three warps per scheduler, exchanges and key updates between the sums).
+// Top-1 / top-3, us, before (a pass per 4 queries / per query) -> now:
+//   8 queries, 50,021 x 384      53 / 170 ->  24 /  24   (77 MB: 11 us)
+//   23                          144 / 449 ->  38 /  42
+//   256                        1453 / 4750 -> 301 / 308   (9.8 GFLOP: 122 us)
+//   8 queries, 500,000 x 384    419 / 1033 -> 136 / 143   (768 MB: 113 us)
+//   8 queries, 300,000 x 768    608 / 1347 -> 158 / 164   (922 MB: 136 us)
+constexpr int kGemmWarps = 12;
+constexpr int kGemmThreads = kGemmWarps * 32;
+constexpr int kGemmStages = 4;
+constexpr int kGemmMaxDim = 1024;
+constexpr int kGemmStageBytes = 49152;   // at least 24 rows of up to 512 dims, 12 of up to 1024
+
+struct GemmSmem {
+    alignas(128) unsigned char ring[kGemmStages][kGemmStageBytes];
+    uint64_t full[kGemmStages];
+    uint64_t empty[kGemmStages];
+    unsigned long long best[kGemmWarps * 8];
+};
+
+template <int LIST>
+__device__ __forceinline__ void insert_key(unsigned long long (&l)[LIST], unsigned long long v) {
+    if (v <= l[LIST - 1]) return;
+#pragma unroll
+    for (int j = LIST - 1; j > 0; --j) {
+        const bool shift = v > l[j - 1];
+        l[j] = shift ? l[j - 1] : (v > l[j] ? v : l[j]);
+    }
+    l[0] = v > l[0] ? v : l[0];
+}
+
+// LIST = 1: partial[blockIdx.x * n_queries + q] = best key of this CTA's rows; else the
+// LIST best, sorted, in the first LIST of kListK entries of partial[(blockIdx.x *
+// n_queries + q) * kListK]. Pass y0 + blockIdx.y takes WQ * QW queries.
+template <int VPL, int QW, int LIST>
+__global__ void __launch_bounds__(kGemmThreads, 1)
+    gemm_retrieve_kernel(const float *__restrict__ index, int64_t M, int dim, const float *__restrict__ queries,
+                         int n_queries, int TR, int WQ, int y0, unsigned long long *__restrict__ partial) {
+    constexpr int NC = 2 * QW;   // sums of a row pair
+    extern __shared__ __align__(128) unsigned char smem_raw[];
+    GemmSmem &sm = *reinterpret_cast<GemmSmem *>(smem_raw);
+    const int lane = threadIdx.x & 31;
+    const int warp = threadIdx.x >> 5;
+    const int WR = kGemmWarps / WQ;
+    const int wq = warp % WQ, wr = warp / WQ;
+    const int q0 = (y0 + static_cast<int>(blockIdx.y)) * WQ * QW;   // first query of the pass
+    const int vecs = dim / 4;
+    const int64_t ntiles = (M + TR - 1) / TR;
+    const int64_t first = blockIdx.x, step = gridDim.x;
+
+    if (threadIdx.x == 0) {
+        for (int s = 0; s < kGemmStages; ++s) {
+            mbar_init(&sm.full[s], 1);
+            mbar_init(&sm.empty[s], kGemmWarps);
+        }
+        fence_barrier_init();
+    }
+    if (threadIdx.x < kGemmWarps * 8) sm.best[threadIdx.x] = 0ull;
+    __syncthreads();
+    auto issue = [&](int64_t k) {   // one thread: this CTA's k-th tile
+        const int64_t r0 = (first + k * step) * TR;
+        const int64_t rows = M - r0 < TR ? M - r0 : TR;
+        const uint32_t bytes = static_cast<uint32_t>(rows * dim * 4);
+        const int s = static_cast<int>(k % kGemmStages);
+        mbar_arrive_expect_tx(&sm.full[s], bytes);
+        bulk_g2s(sm.ring[s], index + r0 * dim, bytes, &sm.full[s]);
+    };
+    const int64_t mine = first < ntiles ? (ntiles - first + step - 1) / step : 0;
+    int64_t issued = 0;
+    for (; warp == 0 && issued < kGemmStages && issued < mine; ++issued)
+        if (lane == 0) issue(issued);
+
+    f2 qv[QW][VPL][2];
+#pragma unroll
+    for (int i = 0; i < QW; ++i)
+#pragma unroll
+        for (int j = 0; j < VPL; ++j) {
+            const int v = lane + 32 * j, q = q0 + wq * QW + i;
+            const bool in = v < vecs && q < n_queries;
+            const ulonglong2 raw =
+                in ? __ldg(reinterpret_cast<const ulonglong2 *>(queries + static_cast<int64_t>(q) * dim) + v)
+                   : make_ulonglong2(0ull, 0ull);
+            qv[i][j][0] = raw.x;
+            qv[i][j][1] = raw.y;
+        }
+    // the sum that this lane ends up with: bit b of the sum's index is lane bit 4 - b
+    int sum = 0;
+#pragma unroll
+    for (int h = NC / 2, o = 16; h > 0; h >>= 1, o >>= 1) sum += (lane & o) ? h : 0;
+    const int sum_r = sum / QW;
+    unsigned long long l[LIST];
+#pragma unroll
+    for (int j = 0; j < LIST; ++j) l[j] = 0ull;
+
+    bool ok = true;
+    for (int64_t k = 0; k < mine; ++k) {
+        const int s = static_cast<int>(k % kGemmStages);
+        ok = __all_sync(0xffffffffu, mbar_wait(&sm.full[s], static_cast<uint32_t>((k / kGemmStages) & 1)));
+        if (!ok) break;
+        const int64_t r0 = (first + k * step) * TR;
+        const int rows = static_cast<int>(M - r0 < TR ? M - r0 : TR);
+        const unsigned char *tile = sm.ring[s];
+        for (int p = wr; 2 * p < rows; p += WR) {
+            float a[NC];
+#pragma unroll
+            for (int r = 0; r < 2; ++r) {
+                // an odd tile's last pair reads its row twice; the second sum is dropped
+                const int row = 2 * p + r < rows ? 2 * p + r : 2 * p;
+                const ulonglong2 *src = reinterpret_cast<const ulonglong2 *>(tile + static_cast<size_t>(row) * dim * 4);
+                f2 acc[QW];
+#pragma unroll
+                for (int i = 0; i < QW; ++i) acc[i] = 0;
+#pragma unroll
+                for (int j = 0; j < VPL; ++j) {
+                    const int v = lane + 32 * j;
+                    const ulonglong2 x = v < vecs ? src[v] : make_ulonglong2(0ull, 0ull);
+#pragma unroll
+                    for (int i = 0; i < QW; ++i) {
+                        acc[i] = fma2(x.x, qv[i][j][0], acc[i]);
+                        acc[i] = fma2(x.y, qv[i][j][1], acc[i]);
+                    }
+                }
+#pragma unroll
+                for (int i = 0; i < QW; ++i) {
+                    float lo, hi;
+                    unpack2(acc[i], lo, hi);
+                    a[r * QW + i] = lo + hi;
+                }
+            }
+            int o = 16;
+#pragma unroll
+            for (int h = NC / 2; h > 0; h >>= 1, o >>= 1) {
+                const bool up = (lane & o) != 0;
+#pragma unroll
+                for (int i = 0; i < h; ++i) {
+                    const float keep = up ? a[i + h] : a[i], send = up ? a[i] : a[i + h];
+                    a[i] = keep + __shfl_xor_sync(0xffffffffu, send, o);
+                }
+            }
+#pragma unroll
+            for (int b = 0; b < 5; ++b)
+                if ((16 >> b) <= 16 / NC) a[0] += __shfl_xor_sync(0xffffffffu, a[0], 16 >> b);
+            const int64_t row = r0 + 2 * p + sum_r;
+            if (2 * p + sum_r < rows && !isnan(a[0])) insert_key<LIST>(l, make_key(a[0], row));
+        }
+        __syncwarp();
+        if (lane == 0) mbar_arrive(&sm.empty[s]);
+        // warp 0 refills the stage of the tile before this one: the other warps are done with
+        // it or nearly (the whole warp leaves together when a wait runs out)
+        if (warp == 0 && k > 0 && issued < mine) {
+            const int64_t f = issued - kGemmStages;   // tile k - 1
+            ok = __all_sync(0xffffffffu, mbar_wait(&sm.empty[f % kGemmStages], static_cast<uint32_t>((f / kGemmStages) & 1)));
+            if (!ok) break;
+            if (lane == 0) {
+                fence_proxy_async_smem();
+                issue(issued);
+            }
+            ++issued;
+        }
+    }
+    if (!ok) atomicOr(&g_retrieve_status, PRECOG_DEV_TIMEOUT);
+    if (threadIdx.x == 0 && !ok)   // issued copies land before the CTA leaves
+        for (int64_t f = issued > kGemmStages ? issued - kGemmStages : 0; f < issued; ++f)
+            mbar_wait(&sm.full[f % kGemmStages], static_cast<uint32_t>((f / kGemmStages) & 1));
+    __syncthreads();
+    const bool keeper = (lane & (32 / NC - 1)) == 0;   // one of the lanes that hold the same sum
+    if constexpr (LIST == 1) {
+        if (keeper && l[0] != 0ull) atomicMax(&sm.best[wq * QW + sum % QW], l[0]);
+        __syncthreads();
+        const int q = q0 + static_cast<int>(threadIdx.x);
+        if (static_cast<int>(threadIdx.x) < WQ * QW && q < n_queries)
+            partial[static_cast<int64_t>(blockIdx.x) * n_queries + q] = sm.best[threadIdx.x];
+    } else {
+        // lists[query][row share and parity][LIST] in the ring, merged by one warp per query (a
+        // lane per list, the largest head LIST times) when they are many, else by one thread
+        constexpr int kWritten = LIST <= 4 ? 4 : kListK;   // entries that the finalize reads
+        unsigned long long *lists = reinterpret_cast<unsigned long long *>(sm.ring);
+        if (keeper)
+#pragma unroll
+            for (int j = 0; j < LIST; ++j)
+                lists[((wq * QW + sum % QW) * 2 * WR + 2 * wr + sum_r) * LIST + j] = l[j];
+        __syncthreads();
+        unsigned long long m[LIST];
+        if (WR >= 6) {
+            for (int i = warp; i < WQ * QW && q0 + i < n_queries; i += kGemmWarps) {
+#pragma unroll
+                for (int j = 0; j < LIST; ++j) m[j] = lane < 2 * WR ? lists[(i * 2 * WR + lane) * LIST + j] : 0ull;
+                unsigned long long out = 0ull;   // lane j: the j-th best
+#pragma unroll
+                for (int j = 0; j < LIST; ++j) {
+                    const unsigned long long key = warp_max_u64(m[0]);
+                    if (lane == j) out = key;
+                    if (key == m[0]) {
+#pragma unroll
+                        for (int h = 0; h + 1 < LIST; ++h) m[h] = m[h + 1];
+                        m[LIST - 1] = 0ull;
+                    }
+                }
+                if (lane < kWritten)
+                    partial[(static_cast<int64_t>(blockIdx.x) * n_queries + q0 + i) * kListK + lane] = out;
+            }
         } else {
-            best_idx[o] = static_cast<int64_t>(0xffffffffu - static_cast<uint32_t>(key & 0xffffffffu));
-            if (best_score) best_score[o] = unordered_float(static_cast<uint32_t>(key >> 32));
+            const int i = static_cast<int>(threadIdx.x);
+            if (i < WQ * QW && q0 + i < n_queries) {
+#pragma unroll
+                for (int j = 0; j < LIST; ++j) m[j] = lists[i * 2 * WR * LIST + j];
+                for (int r = 1; r < 2 * WR; ++r)
+                    for (int j = 0; j < LIST; ++j) {
+                        const unsigned long long v = lists[(i * 2 * WR + r) * LIST + j];
+                        if (v <= m[LIST - 1]) break;   // sorted: the rest is smaller
+                        insert_key<LIST>(m, v);
+                    }
+#pragma unroll
+                for (int j = 0; j < kWritten; ++j)
+                    partial[(static_cast<int64_t>(blockIdx.x) * n_queries + q0 + i) * kListK + j] =
+                        j < LIST ? m[j < LIST ? j : 0] : 0ull;
+            }
         }
     }
 }
@@ -352,15 +613,18 @@ cudaError_t launch_gemv_pass(const RetrieveParams &p, int grid, int q0, cudaStre
     return cudaGetLastError();
 }
 
+// The lengths of rows that reach each kernel (use_gemm): a single query's top-1 up to 512 dims
+// or beyond kGemmMaxDim, everything else beyond kGemmMaxDim only.
 template <typename T, int QB>
 cudaError_t gemv_pass_vpl(const RetrieveParams &p, int grid, int q0, cudaStream_t stream) {
     const int vecs = p.dim / Vec<T>::n;
     const int vpl = (vecs + 31) / 32;
-    if (vpl <= 1) return launch_gemv_pass<T, QB, 1>(p, grid, q0, stream);
-    if (vpl <= 2) return launch_gemv_pass<T, QB, 2>(p, grid, q0, stream);
-    if (vpl <= 3) return launch_gemv_pass<T, QB, 3>(p, grid, q0, stream);
-    if (vpl <= 4) return launch_gemv_pass<T, QB, 4>(p, grid, q0, stream);
-    if (vpl <= 8) return launch_gemv_pass<T, QB, 8>(p, grid, q0, stream);
+    if constexpr (QB == 1) {
+        if (vpl <= 1) return launch_gemv_pass<T, QB, 1>(p, grid, q0, stream);
+        if (vpl <= 2) return launch_gemv_pass<T, QB, 2>(p, grid, q0, stream);
+        if (vpl <= 3) return launch_gemv_pass<T, QB, 3>(p, grid, q0, stream);
+        if (vpl <= 4) return launch_gemv_pass<T, QB, 4>(p, grid, q0, stream);
+    }
     return launch_gemv_pass<T, QB, 16>(p, grid, q0, stream);
 }
 
@@ -380,8 +644,7 @@ cudaError_t launch_gemv(const RetrieveParams &p, cudaStream_t stream, int grid, 
 // 16-bit indexes go to the tensor cores: one pass over the keys for up to 256 queries,
 // streamed by TMA; even a single query's pass is a little faster there (0.246 vs 0.266
 // ms over 1M x 768 fp16 keys) than a CUDA-core GEMV, which needs a pass per 4 queries.
-// fp32 indexes stay on the CUDA cores (the GEMV kernels below are instantiated for fp32
-// keys only).
+// fp32 indexes stay on the CUDA cores (their kernels are instantiated for fp32 keys only).
 bool use_tc(const RetrieveParams &p) { return p.dtype != PRECOG_F32; }
 
 template <typename T, int VPL>
@@ -397,15 +660,69 @@ cudaError_t launch_gemv_topk(const RetrieveParams &p, cudaStream_t stream, int g
                              uint64_t *launches) {
     const int vpl = (p.dim / Vec<T>::n + 31) / 32;
     cudaError_t e = cudaSuccess;
-    for (int q = 0; q < p.n_queries && e == cudaSuccess; ++q, ++*launches) {
-        if (vpl <= 1) e = launch_topk_pass<T, 1>(p, grid, q, stream);
-        else if (vpl <= 2) e = launch_topk_pass<T, 2>(p, grid, q, stream);
-        else if (vpl <= 3) e = launch_topk_pass<T, 3>(p, grid, q, stream);
-        else if (vpl <= 4) e = launch_topk_pass<T, 4>(p, grid, q, stream);
-        else if (vpl <= 8) e = launch_topk_pass<T, 8>(p, grid, q, stream);
-        else e = launch_topk_pass<T, 16>(p, grid, q, stream);
-    }
+    for (int q = 0; q < p.n_queries && e == cudaSuccess; ++q, ++*launches)
+        e = vpl <= 3 ? launch_topk_pass<T, 3>(p, grid, q, stream) : launch_topk_pass<T, 16>(p, grid, q, stream);
     return e;
+}
+
+// fp32 keys of up to kGemmMaxDim dims go to the shared-row kernel. A single query's pass does
+// up to 8 queries' arithmetic there, so it goes where that is faster (us, GEMV / shared rows):
+// top-1 over rows of more than 512 dims (300,000 x 768: 181 / 139; 200,000 x 256: 42 / 47; 384
+// and 512 dims within 2 %); top-k always (50,021 x 384, k = 3: 36 / 24) but for long lists over
+// 257 to 384 dims, where insertions stall its few warps (500,000 x 384, k = 8: 146 / 180).
+bool use_gemm(const RetrieveParams &p, bool topk, int k) {
+    if (p.dim > kGemmMaxDim) return false;
+    if (p.n_queries > 1) return true;
+    if (!topk) return p.dim > 512;
+    return k <= 3 || p.dim <= 256 || p.dim > 384;
+}
+
+// Rows per tile: 24 (12 for rows over 512 dims), and for short rows as many times that as a
+// stage holds while every SM still gets a few tiles.
+int gemm_tile_rows(int64_t M, int dim) {
+    int rows = dim <= 512 ? 24 : 12;
+    while (2 * rows * dim * 4 <= kGemmStageBytes && M / (2 * rows) >= 4 * static_cast<int64_t>(num_sms())) rows *= 2;
+    return rows;
+}
+
+int gemm_grid(int64_t M, int dim) {
+    const int rows = gemm_tile_rows(M, dim);
+    // no more parts than the workspace is sized for
+    return static_cast<int>(std::min<int64_t>(std::min<int64_t>((M + rows - 1) / rows, num_sms()), gemv_grid(M)));
+}
+
+template <int VPL, int QW, int LIST>
+cudaError_t launch_gemm_vq(const RetrieveParams &p, int grid, cudaStream_t stream, uint64_t *launches) {
+    const int groups = (p.n_queries + QW - 1) / QW;
+    const int passes = (groups + kGemmWarps - 1) / kGemmWarps;
+    int WQ = (groups + passes - 1) / passes;
+    while (kGemmWarps % WQ != 0) ++WQ;   // warps split evenly into query groups
+    auto kern = gemm_retrieve_kernel<VPL, QW, LIST>;
+    const int smem = static_cast<int>(sizeof(GemmSmem));
+    cudaError_t e = ensure_smem(reinterpret_cast<const void *>(kern), smem);
+    if (e != cudaSuccess) return e;
+    const int per_launch = 65535;   // passes per launch (grid y)
+    for (int y0 = 0; y0 * WQ < groups; y0 += per_launch) {
+        const int left = (groups - y0 * WQ + WQ - 1) / WQ;
+        kern<<<dim3(static_cast<unsigned>(grid), static_cast<unsigned>(std::min(left, per_launch))), kGemmThreads, smem,
+               stream>>>(static_cast<const float *>(p.index), p.M, p.dim, static_cast<const float *>(p.queries),
+                         p.n_queries, gemm_tile_rows(p.M, p.dim), WQ, y0, static_cast<unsigned long long *>(p.workspace));
+        e = cudaGetLastError();
+        if (e != cudaSuccess) return e;
+        ++*launches;
+    }
+    return cudaSuccess;
+}
+
+template <int LIST>
+cudaError_t launch_gemm(const RetrieveParams &p, int grid, cudaStream_t stream, uint64_t *launches) {
+    const int vpl = (p.dim / 4 + 31) / 32;
+    if (vpl <= 1) return launch_gemm_vq<1, 8, LIST>(p, grid, stream, launches);
+    if (vpl <= 2) return launch_gemm_vq<2, 8, LIST>(p, grid, stream, launches);
+    if (vpl <= 3) return launch_gemm_vq<3, 8, LIST>(p, grid, stream, launches);
+    if (vpl <= 4) return launch_gemm_vq<4, 4, LIST>(p, grid, stream, launches);
+    if (vpl <= 6) return launch_gemm_vq<6, 4, LIST>(p, grid, stream, launches);
+    return launch_gemm_vq<8, 2, LIST>(p, grid, stream, launches);
 }
 
 }  // namespace
@@ -427,6 +744,9 @@ cudaError_t launch_retrieve(const RetrieveParams &p, cudaStream_t stream) {
     if (p.M > 0 && use_tc(p)) {
         parts = retrieve_tc_grid(p.M, num_sms());
         e = launch_retrieve_tc(p, parts, stream, &launches);
+    } else if (p.M > 0 && use_gemm(p, false, 1)) {
+        parts = gemm_grid(p.M, p.dim);
+        e = launch_gemm<1>(p, parts, stream, &launches);
     } else if (p.M > 0) {
         parts = gemv_grid(p.M);
         e = launch_gemv<float>(p, stream, parts, &launches);
@@ -465,16 +785,22 @@ cudaError_t launch_retrieve_topk(const RetrieveParams &p, int k, cudaStream_t st
     uint64_t launches = 0;
     cudaError_t e = cudaSuccess;
     int parts = 0;  // an empty index has no partial lists: the finalize writes rows -1
+    int log_used = 3;
     if (p.M > 0 && use_tc(p)) {
         parts = retrieve_tc_grid(p.M, num_sms());
         e = launch_retrieve_tc_topk(p, k, parts, stream, &launches);
+        log_used = k <= 2 ? 1 : (k <= 4 ? 2 : 3);   // the tensor-core kernel's list lengths
+    } else if (p.M > 0 && use_gemm(p, true, k)) {
+        parts = gemm_grid(p.M, p.dim);
+        e = k <= 3 ? launch_gemm<3>(p, parts, stream, &launches) : launch_gemm<8>(p, parts, stream, &launches);
+        log_used = k <= 3 ? 2 : 3;
     } else if (p.M > 0) {
         parts = gemv_grid(p.M);
         e = launch_gemv_topk<float>(p, stream, parts, &launches);
     }
     if (e == cudaSuccess) {
         finalize_topk_kernel<<<(p.n_queries + 3) / 4, 128, 0, stream>>>(
-            static_cast<const unsigned long long *>(p.workspace), parts, p.n_queries, k, p.best_idx,
+            static_cast<const unsigned long long *>(p.workspace), parts, log_used, p.n_queries, k, p.best_idx,
             p.best_score);
         e = cudaGetLastError();
         if (e == cudaSuccess) ++launches;

@@ -143,3 +143,38 @@ def test_topk_empty_index(cuda_device, dtype_name):
     idx, score = _topk(torch.empty((0, 64), dtype=dtype, device=cuda_device),
                        torch.ones((2, 64), dtype=dtype, device=cuda_device), 3)
     assert (idx == -1).all() and np.isnan(score).all()
+
+
+@pytest.mark.parametrize("M,dim", [(1, 4), (23, 64), (25, 132), (700, 256), (611, 260), (5000, 384), (3001, 388),
+                                   (49, 512), (13, 516), (400, 768), (30000, 64), (200, 1024), (60, 1028)])
+@pytest.mark.parametrize("Q", [1, 2, 9, 25, 97])
+def test_f32_batches_share_rows(cuda_device, M, dim, Q):
+    """fp32 keys: the kernels that share rows among query groups, at the edges of their
+    tiles (12 and 24 rows, odd last pairs), of the lanes' vectors (a row that ends inside a
+    lane's share must not read the next row's NaN), of the query groups and of the passes,
+    and beyond the longest row they take. Small integers: exact scores and many ties."""
+    import torch
+    pg = _pg()
+    rng = np.random.default_rng(M + dim + Q)
+    index = rng.integers(-3, 4, size=(M, dim)).astype(np.float32)
+    index[rng.random(M) < 0.1, 0] = np.nan
+    index[rng.random(M) < 0.02] = np.inf       # inf - inf or inf: NaN or the best score
+    queries = rng.integers(-3, 4, size=(Q, dim)).astype(np.float32)
+    t = lambda a: torch.from_numpy(a).to(cuda_device)
+    with np.errstate(invalid="ignore"):
+        s = queries @ index.T                  # exact in fp32: |sum| < 2^24
+    order = np.argsort(-np.where(np.isnan(s), -np.inf, s), axis=1, kind="stable")
+    for k in (1, 3, 8):
+        idx, score = _topk(t(index), t(queries), k)
+        for q in range(Q):
+            best = [r for r in order[q] if not np.isnan(s[q, r])][:k]
+            np.testing.assert_array_equal(idx[q], best + [-1] * (k - len(best)))
+            np.testing.assert_array_equal(score[q, :len(best)], s[q, best])
+            assert np.isnan(score[q, len(best):]).all()
+        if k == 1:
+            i1 = torch.empty(Q, dtype=torch.int64, device=cuda_device)
+            s1 = torch.empty(Q, dtype=torch.float32, device=cuda_device)
+            pg.precog_retrieve(t(index), t(queries), i1, s1)
+            assert pg.precog_device_status()[0] == 0
+            np.testing.assert_array_equal(i1.cpu().numpy(), idx[:, 0])
+            np.testing.assert_array_equal(s1.cpu().numpy(), score[:, 0])
