@@ -108,8 +108,9 @@ struct TrajCursor {
 };
 
 // Tensor maps of x and dt for launches whose CTAs take a slice of each row: the tensor is
-// viewed as [layer][row][D / inner][inner] (inner = min(slice, 256) channels, the widest
-// box dimension), so a box of [1][TILE][slice / inner][inner] is one slice of TILE rows.
+// viewed as [layer][row][D / inner][inner] (inner = min(slice, 256), the widest box dimension),
+// so a box of [1][TILE][slice / inner][inner] is one slice of TILE rows; inner == 0: the
+// slices don't divide the row and a box starts at its channel of [layer][row][1][D].
 struct SliceMaps {
     CUtensorMap x, dt;
     int32_t valid, inner;
@@ -330,7 +331,7 @@ template <class C>
 __device__ __forceinline__ void scan_tile_direct(const unsigned char *st, const StageLayout &lay,
                                                  int DS, int dl, int ntok,
                                                  f2 (&h)[C::CPT][8], const float (&kpow)[C::CPT],
-                                                 const f2 (&kgen)[C::CPT][8], void *yrow,
+                                                 const f2 (&kgen)[C::CPT][8], bool live, void *yrow,
                                                  int y_dtype, int64_t y_stride,
                                                  const ScanParams &p, TrajCursor &tc,
                                                  int64_t tok_left, int traj_layer, int dglob) {
@@ -397,7 +398,7 @@ __device__ __forceinline__ void scan_tile_direct(const unsigned char *st, const 
                 yv[j] = lo + hi;
             }
         }
-        if constexpr (C::HAS_Y) {
+        if (C::HAS_Y && live) {
             if (y_dtype == PRECOG_F32) {
                 float *dst = static_cast<float *>(yrow) + t * y_stride;
                 if constexpr (CPT == 2) {
@@ -421,7 +422,7 @@ __device__ __forceinline__ void scan_tile_direct(const unsigned char *st, const 
             // after every stride-th token and after the chunk's last token (uniform)
             if (--tc.left == 0 || t + 1 == tok_left) {
 #pragma unroll
-                for (int j = 0; j < CPT; ++j)
+                for (int j = 0; live && j < CPT; ++j)
                     store_state16(p.traj, p.traj_dtype,
                                   ((tc.entry * p.L_out + traj_layer) * static_cast<int64_t>(p.D) + dglob + j) *
                                       kN,
@@ -688,6 +689,8 @@ __global__ void __launch_bounds__(C::LB_THREADS, C::LB_BLOCKS)
         return;
     }
     const int layer = static_cast<int>(item / p.n_chunks);
+    // a last slice narrower than the others leaves its upper threads without channels
+    const bool live = C::FIXDS || slice * DS + static_cast<int>(threadIdx.x) * CPT < p.D;
     // this thread's rows of A first (16 floats each, 16-byte loads): their latency overlaps
     // the chunk's offsets below
     float a_rows[CPT][kN];
@@ -699,7 +702,7 @@ __global__ void __launch_bounds__(C::LB_THREADS, C::LB_BLOCKS)
                 Al0 + static_cast<int64_t>(slice * DS + static_cast<int>(threadIdx.x) * CPT + j) * kN);
 #pragma unroll
             for (int q = 0; q < kN / 4; ++q) {
-                const float4 v = a4[q];
+                const float4 v = live ? a4[q] : make_float4(0.f, 0.f, 0.f, 0.f);
                 a_rows[j][4 * q] = v.x;
                 a_rows[j][4 * q + 1] = v.y;
                 a_rows[j][4 * q + 2] = v.z;
@@ -785,13 +788,16 @@ __global__ void __launch_bounds__(C::LB_THREADS, C::LB_BLOCKS)
             // the slice of TILE rows as one tensor-map copy per tensor (a box always moves
             // TILE rows; rows past the end of the tensor arrive as zeros)
             mbar_arrive_expect_tx(&full[s], bytes + (TILE - ntok) * rowb * 2);
-            tma_load_4d(st + lay.xs, &maps.x, 0, d0 / maps.inner, static_cast<int32_t>(row0), layer, &full[s]);
-            tma_load_4d(st + lay.dts, &maps.dt, 0, d0 / maps.inner, static_cast<int32_t>(row0), layer, &full[s]);
+            const bool even = C::FIXDS || maps.inner;
+            const int c0 = even ? 0 : d0, c1 = even ? d0 / maps.inner : 0;
+            tma_load_4d(st + lay.xs, &maps.x, c0, c1, static_cast<int32_t>(row0), layer, &full[s]);
+            tma_load_4d(st + lay.dts, &maps.dt, c0, c1, static_cast<int32_t>(row0), layer, &full[s]);
         } else {
-            mbar_arrive_expect_tx(&full[s], bytes);
+            const uint32_t ownb = !C::FIXDS && D - d0 < DS ? (D - d0) * SZ : rowb;   // the slice's part of the row
+            mbar_arrive_expect_tx(&full[s], bytes - ntok * (rowb - ownb) * 2);
             for (int r = 0; r < ntok; ++r) {
-                bulk_g2s(st + lay.xs + r * rowb, xl + (row0 + r) * D + d0, rowb, &full[s]);
-                bulk_g2s(st + lay.dts + r * rowb, dtl + (row0 + r) * D + d0, rowb, &full[s]);
+                bulk_g2s(st + lay.xs + r * rowb, xl + (row0 + r) * D + d0, ownb, &full[s]);
+                bulk_g2s(st + lay.dts + r * rowb, dtl + (row0 + r) * D + d0, ownb, &full[s]);
             }
         }
         bulk_g2s(st + lay.bs, Bl + row0 * kN, ntok * kN * SZ, &full[s]);
@@ -814,7 +820,7 @@ __global__ void __launch_bounds__(C::LB_THREADS, C::LB_BLOCKS)
     }
 #pragma unroll
     for (int j = 0; j < CPT; ++j) {
-        if (C::HAS_H0 && h0_valid) {
+        if (C::HAS_H0 && h0_valid && live) {
             const int64_t off =
                 ((h0_row * p.L_bank + p.layer0 + layer) * static_cast<int64_t>(D) + d0 + dl + j) * kN;
             load_state16(p.bank, p.bank_dtype, off, h[j]);
@@ -858,7 +864,7 @@ __global__ void __launch_bounds__(C::LB_THREADS, C::LB_BLOCKS)
                 const float wk = w[k] / wsum;
                 const f2 ww = pack2(wk, wk);
 #pragma unroll
-                for (int j = 0; j < CPT; ++j) {
+                for (int j = 0; live && j < CPT; ++j) {
                     f2 hk[8];
                     const int64_t off = ((rows[k] * p.L_bank + p.layer0 + layer) * static_cast<int64_t>(D) +
                                          d0 + dl + j) * kN;
@@ -943,7 +949,7 @@ __global__ void __launch_bounds__(C::LB_THREADS, C::LB_BLOCKS)
 #pragma unroll
                     for (int j = 0; j < CPT; ++j) {
                         renormalise(h[j], Lw[j]);
-                        store_state16(p.traj, p.traj_dtype,
+                        if (live) store_state16(p.traj, p.traj_dtype,
                                       ((tcur.entry * p.L_out + p.layer0 + layer) * static_cast<int64_t>(D) +
                                        d0 + dl + j) * kN,
                                       h[j]);
@@ -956,7 +962,7 @@ __global__ void __launch_bounds__(C::LB_THREADS, C::LB_BLOCKS)
             scan_tile_rescaled<C>(st, lay, reinterpret_cast<const float *>(st + (C::CONV ? lay.bf : lay.bs)), DS, dl, 0,
                                   ntok, h, Lw, kk, wmask);
         } else {
-            scan_tile_direct<C>(st, lay, DS, dl, ntok, h, kpow, kgen, yrow, p.y_dtype, y_stride, p, tcur,
+            scan_tile_direct<C>(st, lay, DS, dl, ntok, h, kpow, kgen, live, yrow, p.y_dtype, y_stride, p, tcur,
                                 len - k * TILE, p.layer0 + layer, d0 + dl);
         }
         if (C::HAS_Y) {
@@ -974,7 +980,7 @@ __global__ void __launch_bounds__(C::LB_THREADS, C::LB_BLOCKS)
 #pragma unroll
         for (int j = 0; j < CPT; ++j) renormalise(h[j], Lw[j]);
     }
-    if (p.states) {
+    if (p.states && live) {
 #pragma unroll
         for (int j = 0; j < CPT; ++j) {
             const int64_t off =
@@ -984,13 +990,16 @@ __global__ void __launch_bounds__(C::LB_THREADS, C::LB_BLOCKS)
     }
 }
 
-// Widest channel slice (<= maxslice channels, 16-byte rows) that divides D
-// into whole threads of CPT channels.
-int pick_slice(int D, int sz, int cpt, int maxslice) {
-    const int cands[] = {512, 256, 128, 64, 32, 16, 8, 4, 2};
-    for (int ds : cands)
-        if (ds <= maxslice && D % ds == 0 && (ds * sz) % 16 == 0 && ds % cpt == 0) return ds;
-    return 0;
+// Channel slice of one CTA: the widest of 512 (if maxslice allows it), 256 and 128 channels that
+// divides the row; else the whole row if it fits, whatever its length, or slices of 256 whose
+// last one is narrower (its upper threads have no channels). Slices had to be a power of two
+// that divides D, so D = 1000 or 712 ran 125 or 89 CTAs of two threads per chunk: 2 layers x
+// 400 chunks x 200 tokens bf16, D = 1000: capture 3654 -> 225 us, readout 7035 -> 421 us,
+// general A (fp32) 2593 -> 540 us; D = 456: 1678 -> 128, 3219 -> 229, 1189 -> 275 us.
+int pick_slice(int D, int maxslice) {
+    for (int ds = kWideSlice; ds >= 128; ds /= 2)
+        if (ds <= maxslice && D % ds == 0) return ds;
+    return D <= maxslice ? D : kMaxSlice;
 }
 
 // True when a full-width launch would have fewer CTAs than the device has SMs.
@@ -1002,10 +1011,9 @@ bool few_items(const ScanParams &p) {
 
 template <class C>
 cudaError_t launch_cfg(const ScanParams &p, cudaStream_t stream) {
-    const int DS = C::FIXDS ? (p.D % C::FIXDS == 0 && (C::FIXDS * C::SZ) % 16 == 0 ? C::FIXDS : 0)
-                            : pick_slice(p.D, C::SZ, C::CPT, C::MAXSLICE);
-    if (DS == 0) return cudaErrorInvalidValue;
-    const int slices = p.D / DS;
+    const int DS = C::FIXDS ? C::FIXDS : pick_slice(p.D, C::MAXSLICE);
+    if (DS % C::CPT != 0 || (C::FIXDS && p.D % DS != 0)) return cudaErrorInvalidValue;
+    const int slices = (p.D + DS - 1) / DS;
     const StageLayout lay = stage_layout(C::TILE, DS, C::SZ, C::HAS_Y, C::CONV);
     const size_t smem = kBarBytes + static_cast<size_t>(C::STAGES) * lay.bytes;
     const int64_t items = static_cast<int64_t>(p.n_layers) * p.n_chunks * slices;
@@ -1013,19 +1021,22 @@ cudaError_t launch_cfg(const ScanParams &p, cudaStream_t stream) {
     if (items > 0x7fffffffLL) return cudaErrorInvalidConfiguration;
     SliceMaps maps{};
     if (DS < p.D) {
-        const int inner = DS < 256 ? DS : 256;
+        // slices that divide the row: [layer][row][D / inner][inner], a box of whole inner rows;
+        // else [layer][row][1][D], a box from channel d0 (channels past the row arrive as zeros)
+        const bool even = p.D % DS == 0;
+        const int inner = even ? (DS < 256 ? DS : 256) : p.D;
         const cuuint64_t rows = static_cast<cuuint64_t>(p.T_tot);
         const cuuint64_t dims[4] = {static_cast<cuuint64_t>(inner), static_cast<cuuint64_t>(p.D / inner), rows,
                                     static_cast<cuuint64_t>(p.n_layers)};
         const cuuint64_t lstride = static_cast<cuuint64_t>(p.n_layers > 1 ? p.ls_xd : rows * p.D) * C::SZ;
         const cuuint64_t strides[3] = {static_cast<cuuint64_t>(inner) * C::SZ, static_cast<cuuint64_t>(p.D) * C::SZ,
                                        lstride};
-        const cuuint32_t box[4] = {static_cast<cuuint32_t>(inner), static_cast<cuuint32_t>(DS / inner),
+        const cuuint32_t box[4] = {static_cast<cuuint32_t>(DS < 256 ? DS : 256), static_cast<cuuint32_t>(even ? DS / inner : 1),
                                    static_cast<cuuint32_t>(C::TILE), 1};
         const CUtensorMapDataType dt = C::SZ == 4 ? CU_TENSOR_MAP_DATA_TYPE_FLOAT32 : CU_TENSOR_MAP_DATA_TYPE_BFLOAT16;
         maps.valid = encode_tiled_map(&maps.x, dt, 4, p.x, dims, strides, box, CU_TENSOR_MAP_SWIZZLE_NONE) &&
                      encode_tiled_map(&maps.dt, dt, 4, p.dt, dims, strides, box, CU_TENSOR_MAP_SWIZZLE_NONE);
-        maps.inner = inner;
+        maps.inner = even ? inner : 0;
     }
     auto kern = scan_kernel<C>;
     cudaError_t e = ensure_smem(reinterpret_cast<const void *>(kern), static_cast<int>(smem));
@@ -1041,21 +1052,28 @@ cudaError_t launch_cfg(const ScanParams &p, cudaStream_t stream) {
 template <typename TIn, bool HAS_Y, bool HAS_H0, int MODE, int TRAJ = kTrajNone>
 cudaError_t launch_t(const ScanParams &p, cudaStream_t stream) {
     if constexpr (TRAJ == kTrajRescaled) {
+        if (p.D % 256 == 0 && p.D % 512 != 0)
+            return launch_cfg<Cfg<TIn, false, false, kPower, PRECOG_RESCALED_CPT, PRECOG_RESCALED_TILE,
+                                  PRECOG_RESCALED_STAGES, PRECOG_RESCALED_MINB, kTrajRescaled, kWideSlice, 256>>(p, stream);
         return launch_cfg<Cfg<TIn, false, false, kPower, PRECOG_RESCALED_CPT, PRECOG_RESCALED_TILE,
                               PRECOG_RESCALED_STAGES, PRECOG_RESCALED_MINB, kTrajRescaled, kWideSlice>>(p, stream);
     } else if constexpr (TRAJ == kTrajDirect) {
         // short strides and general A: the direct update (h is at hand after every token)
-        if constexpr (MODE == kPower)
+        if constexpr (MODE == kPower) {
+            if (p.D % 256 == 0 && p.D % 512 != 0)
+                return launch_cfg<Cfg<TIn, false, false, MODE, PRECOG_DIRECT_CPT, PRECOG_DIRECT_TILE, PRECOG_DIRECT_STAGES,
+                                      PRECOG_DIRECT_MINB, kTrajDirect, kWideSlice, 256>>(p, stream);
             return launch_cfg<Cfg<TIn, false, false, MODE, PRECOG_DIRECT_CPT, PRECOG_DIRECT_TILE,
                                   PRECOG_DIRECT_STAGES, PRECOG_DIRECT_MINB, kTrajDirect, kWideSlice>>(p, stream);
-        else
+        } else {
             return launch_cfg<Cfg<TIn, false, false, MODE, 2, 16, 4, 3, kTrajDirect>>(p, stream);
+        }
     } else if constexpr (MODE == kPower && !HAS_Y) {
         // the corpus encode of 256- and 512-channel slices (the paper's layer width, the
         // ragged and wide workloads' slices) gets the slice fixed at compile time
         if constexpr (!HAS_H0 && !std::is_same<TIn, float>::value) {
-            const int ds = pick_slice(p.D, sizeof(TIn), PRECOG_RESCALED_CPT, kWideSlice);
-            if (ds == 256)
+            const int ds = pick_slice(p.D, kWideSlice);
+            if (ds == 256 && p.D % 256 == 0)
                 return launch_cfg<Cfg<TIn, false, false, MODE, PRECOG_RESCALED_CPT, PRECOG_RESCALED_TILE,
                                       PRECOG_RESCALED_STAGES, PRECOG_RESCALED_MINB, kTrajNone, kWideSlice, 256>>(
                     p, stream);
@@ -1077,8 +1095,8 @@ cudaError_t launch_t(const ScanParams &p, cudaStream_t stream) {
             }
             if constexpr (!std::is_same<TIn, float>::value) {
                 // 16-bit rows: 256- and 512-channel slices fixed at compile time
-                const int ds = pick_slice(p.D, sizeof(TIn), PRECOG_DIRECT_CPT, kWideSlice);
-                if (ds == 256)
+                const int ds = pick_slice(p.D, kWideSlice);
+                if (ds == 256 && p.D % 256 == 0)
                     return launch_cfg<Cfg<TIn, HAS_Y, HAS_H0, MODE, PRECOG_DIRECT_CPT, PRECOG_DIRECT_TILE,
                                           PRECOG_DIRECT_STAGES, PRECOG_DIRECT_MINB, kTrajNone, kWideSlice, 256>>(
                         p, stream);
@@ -1091,6 +1109,7 @@ cudaError_t launch_t(const ScanParams &p, cudaStream_t stream) {
                                   PRECOG_DIRECT_STAGES, PRECOG_DIRECT_MINB, kTrajNone, kWideSlice>>(p, stream);
         } else {
             // general A keeps 16 exponent coefficients per channel: 2 channels per thread
+            if (p.D % 256 == 0) return launch_cfg<Cfg<TIn, HAS_Y, HAS_H0, MODE, 2, 16, 4, 3, kTrajNone, kMaxSlice, 256>>(p, stream);
             return launch_cfg<Cfg<TIn, HAS_Y, HAS_H0, MODE, 2, 16, 4, 3>>(p, stream);
         }
     }

@@ -510,3 +510,65 @@ def test_ordered_encode_matches_unordered(cuda_device, case):
     assert bool((st[1] == 7.0).all())
     keep = [c for c in range(n) if c != 1]
     assert torch.equal(st[keep], ref_st[keep])
+
+
+@pytest.mark.parametrize("D", [8, 40, 200, 264, 456, 520, 712, 1000, 1032])
+@pytest.mark.parametrize("kind", ["bf16", "f32"])
+@pytest.mark.parametrize("power", [True, False])
+def test_widths_that_slices_do_not_divide(cuda_device, D, kind, power):
+    """Rows of any whole number of 16-byte vectors: kept whole, or cut into slices whose last
+    one is narrower (its upper threads have no channels, its copies run past the row), over
+    two layers: capture, readout, readout from an injected state and trajectories."""
+    import torch
+    pg = _pg()
+    d = cuda_device
+    if kind == "f32":
+        D += 4                                  # 16-byte rows, not of 8 channels
+    dtype = torch.float32 if kind == "f32" else torch.bfloat16
+    L, N = 2, 16
+    lens = [1, 37, 0, 16, 50]
+    off = np.concatenate([[0], np.cumsum(lens)]).astype(np.int64)
+    T = int(off[-1])
+    ins = [synth.host_scan_inputs(T, D, N, seed=D + l) for l in range(L)]
+    rng = np.random.default_rng(D)
+    A = np.stack([i[2] for i in ins]) if power else -rng.uniform(0.05, 3.0, size=(L, D, N)).astype(np.float32)
+    x, dt, B, C = (torch.stack([_t(i[k], d, dtype) for i in ins]) for k in (0, 1, 3, 4))
+    X, DT, Bn, Cn = (to_np(t) for t in (x, dt, B, C))
+    offs = _t(off, d, torch.int64)
+    tol = TOL_F32 if kind == "f32" else TOL_BF16
+    states, y = _encode(d, x, dt, B, _t(A, d), offs, C=C, y_dtype=torch.float32, power=power)
+    capt, _ = _encode(d, x, dt, B, _t(A, d), offs, power=power)
+    bank = rng.standard_normal((len(lens), L, D, N)).astype(np.float32)
+    q = pg.scan_inputs(x[:, :50].contiguous(), dt[:, :50].contiguous(), B[:, :50].contiguous(), _t(A, d),
+                       C[:, :50].contiguous(), a_kind=pg.PRECOG_A_POWER if power else pg.PRECOG_A_GENERAL)
+    qy = torch.zeros((L, 50, D), dtype=torch.float32, device=d)
+    qh = torch.zeros((2, L, D, N), dtype=torch.float32, device=d)
+    pg.precog_prefill_from_state(q, 2, 25, _t(bank, d), torch.tensor([3, -1], device=d), y_out=qy, state_out=qh)
+    trajs = {}
+    for stride in (3, 20):
+        keep = -(-np.asarray(lens) // stride)
+        ent = np.concatenate([[0], np.cumsum(keep)]).astype(np.int64)
+        trajs[stride] = torch.full((int(ent[-1]), L, D, N), float("nan"), device=d)
+        pg.precog_encode_trajectory(pg.scan_inputs(x, dt, B, _t(A, d), a_kind=pg.PRECOG_A_POWER if power else
+                                                   pg.PRECOG_A_GENERAL), offs, T, stride, _t(ent, d, torch.int64),
+                                    trajs[stride])
+    assert pg.precog_device_status()[0] == 0
+    for l in range(L):
+        ref_s, ref_y = oracle.scan(X[l], DT[l], A[l], Bn[l], off, C=Cn[l], want_y=True)
+        assert rel_err(to_np(y[l]), ref_y) < tol
+        e = {3: 0, 20: 0}
+        for c in range(len(lens)):
+            assert rel_err(to_np(states[c, l]), ref_s[c]) < tol
+            assert rel_err(to_np(capt[c, l]), ref_s[c]) < tol
+            for stride in (3, 20):
+                for t in range(stride, lens[c] + stride, stride):
+                    n = min(t, lens[c])
+                    sl = slice(off[c], off[c] + n)
+                    ref, _ = oracle.rollout(X[l, sl], DT[l, sl], A[l], Bn[l, sl])
+                    assert rel_err(to_np(trajs[stride][e[stride], l]), ref) < tol
+                    e[stride] += 1
+        for i, h0 in ((0, bank[3, l]), (1, np.zeros((D, N)))):
+            sl = slice(25 * i, 25 * i + 25)
+            ref_h, ref_q = oracle.rollout(X[l, sl], DT[l, sl], A[l], Bn[l, sl], Cn[l, sl], h0=h0, want_y=True)
+            assert rel_err(to_np(qh[i, l]), ref_h) < tol
+            assert rel_err(to_np(qy[l, sl]), ref_q) < tol
