@@ -1009,6 +1009,11 @@ bool few_items(const ScanParams &p) {
     return static_cast<int64_t>(p.n_layers) * p.n_chunks * slices < sms;
 }
 
+// The same by channels, whatever the number of CTAs they make.
+bool few_channels(const ScanParams &p) {
+    return static_cast<int64_t>(p.n_layers) * p.n_chunks * p.D < static_cast<int64_t>(device_sm_count()) * kMaxSlice;
+}
+
 template <class C>
 cudaError_t launch_cfg(const ScanParams &p, cudaStream_t stream) {
     const int DS = C::FIXDS ? C::FIXDS : pick_slice(p.D, C::MAXSLICE);
@@ -1108,9 +1113,17 @@ cudaError_t launch_t(const ScanParams &p, cudaStream_t stream) {
             return launch_cfg<Cfg<TIn, HAS_Y, HAS_H0, MODE, PRECOG_DIRECT_CPT, PRECOG_DIRECT_TILE,
                                   PRECOG_DIRECT_STAGES, PRECOG_DIRECT_MINB, kTrajNone, kWideSlice>>(p, stream);
         } else {
-            // general A keeps 16 exponent coefficients per channel: 2 channels per thread
-            if (p.D % 256 == 0) return launch_cfg<Cfg<TIn, HAS_Y, HAS_H0, MODE, 2, 16, 4, 3, kTrajNone, kMaxSlice, 256>>(p, stream);
-            return launch_cfg<Cfg<TIn, HAS_Y, HAS_H0, MODE, 2, 16, 4, 3>>(p, stream);
+            // general A keeps 16 exponent coefficients per channel: 2 channels per thread. Two
+            // stages and 128 registers let four CTAs share an SM's SFU (its bound: 16
+            // exponentials per channel-token) where four stages left room for three: 4 layers x
+            // 1000 chunks x 500 tokens fp32 1524 -> 1070 us, bf16 1096 -> 1032, with readout
+            // 2126 -> 1419 and 1721 -> 1443. A readout launch that does not fill the SMs keeps
+            // the deeper ring and the registers (24 x 3 x 500 bf16: 93 us, 102).
+            if constexpr (HAS_Y)
+                if (few_channels(p)) return launch_cfg<Cfg<TIn, HAS_Y, HAS_H0, MODE, 2, 16, 4, 3>>(p, stream);
+            if (p.D % 256 == 0)
+                return launch_cfg<Cfg<TIn, HAS_Y, HAS_H0, MODE, 2, 16, 2, 4, kTrajNone, kMaxSlice, 256>>(p, stream);
+            return launch_cfg<Cfg<TIn, HAS_Y, HAS_H0, MODE, 2, 16, 2, 4>>(p, stream);
         }
     }
 }
