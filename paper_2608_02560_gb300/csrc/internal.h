@@ -49,6 +49,8 @@ struct ScanParams {
     int32_t traj_dtype;
     int64_t traj_stride;
     const int64_t *traj_offsets;  // [n_chunks+1] first entry of each chunk
+    // CTAs that share a chunk's tokens (the split capture; set where it is chosen)
+    int32_t segments;
 };
 
 // Bounded-wait self-test (selftest.cu).

@@ -77,12 +77,14 @@ enum Mode { kGeneral = 0, kPower = 1 };
 constexpr int kTrajNone = 0, kTrajDirect = 1, kTrajRescaled = 2;
 
 template <typename TIn_, bool HAS_Y_, bool HAS_H0_, int MODE_, int CPT_, int TILE_, int STAGES_,
-          int MINB_, int TRAJ_ = kTrajNone, int MAXSLICE_ = kMaxSlice, int FIXDS_ = 0>
+          int MINB_, int TRAJ_ = kTrajNone, int MAXSLICE_ = kMaxSlice, int FIXDS_ = 0, bool SPLIT_ = false>
 struct Cfg {
     using TIn = TIn_;
     // Channel slice known at compile time (0: a launch argument). A constant slice turns
     // the shared-memory row offsets of the time loop into immediates.
     static constexpr int FIXDS = FIXDS_;
+    // A cluster of CTAs per work item, each with a share of the chunk's tokens (see combine).
+    static constexpr bool SPLIT = SPLIT_;
     // Widest channel slice of one CTA. Each CTA stages its slice of every token row; a
     // slice narrower than the row turns the row into separate pieces, and HBM serves
     // short scattered pieces far below its streaming rate, so rows up to 512 channels
@@ -334,14 +336,15 @@ __device__ __forceinline__ void scan_tile_direct(const unsigned char *st, const 
                                                  const f2 (&kgen)[C::CPT][8], bool live, void *yrow,
                                                  int y_dtype, int64_t y_stride,
                                                  const ScanParams &p, TrajCursor &tc,
-                                                 int64_t tok_left, int traj_layer, int dglob) {
+                                                 int64_t tok_left, int traj_layer, int dglob,
+                                                 float (&tot)[C::CPT]) {
     constexpr int CPT = C::CPT;
     const float *bsrc = reinterpret_cast<const float *>(st + (C::CONV ? lay.bf : lay.bs));
     const float *csrc = reinterpret_cast<const float *>(st + (C::CONV ? lay.cf : lay.cs));
     for (int t = 0; t < ntok; ++t) {
         f2 b[8];
         load_b(bsrc, t, b);
-        float xv[CPT], dv[CPT], yv[CPT], uv[CPT];
+        float xv[CPT], dv[CPT], yv[CPT] = {}, uv[CPT];
         uint32_t neg;
         f2 uu2[CPT];   // (u, u) pairs of the 16-bit path, both halves computed
         if constexpr (C::CONV) {
@@ -365,6 +368,10 @@ __device__ __forceinline__ void scan_tile_direct(const unsigned char *st, const 
             load_chan<typename C::TIn, CPT>(st + lay.dts + (t * DS + dl) * C::SZ, dv, neg);
 #pragma unroll
             for (int j = 0; j < CPT; ++j) uv[j] = dv[j] * xv[j];
+        }
+        if constexpr (C::SPLIT) {
+#pragma unroll
+            for (int j = 0; j < CPT; ++j) tot[j] += dv[j];
         }
 #pragma unroll
         for (int j = 0; j < CPT; ++j) {
@@ -560,7 +567,8 @@ template <class C>
 __device__ __forceinline__ void scan_tile_rescaled(const unsigned char *st, const StageLayout &lay,
                                                    const float *bsrc, int DS, int dl, int t0, int ntok,
                                                    f2 (&g)[C::CPT][8], float (&L)[C::CPT],
-                                                   const float (&kk)[C::CPT], unsigned wmask) {
+                                                   const float (&kk)[C::CPT], unsigned wmask,
+                                                   float (&tot)[C::CPT]) {
     constexpr int CPT = C::CPT;
     using TIn = typename C::TIn;
     // 16-bit inputs: dt is kept as raw words across the vote, and u = dt * x is formed
@@ -585,6 +593,12 @@ __device__ __forceinline__ void scan_tile_rescaled(const unsigned char *st, cons
             }
 #pragma unroll
             for (int j = 0; j < CPT; ++j) Lk[k][j] = fmaf(dvk[k][j], kk[j], k ? Lk[k - 1][j] : L[j]);
+        }
+        if constexpr (C::SPLIT) {
+#pragma unroll
+            for (int j = 0; j < CPT; ++j)
+#pragma unroll
+                for (int k = 0; k < kGroup; k += 2) tot[j] += dvk[k][j] + dvk[k + 1][j];
         }
         if constexpr (MIX) neg &= 0x80008000u;
         bool up = false;
@@ -661,11 +675,79 @@ __device__ __forceinline__ void scan_tile_rescaled(const unsigned char *st, cons
         load_b(bsrc, t, b);
         load_chan<TIn, CPT>(st + lay.xs + (t * DS + dl) * C::SZ, xv, n0);
         load_chan<TIn, CPT>(st + lay.dts + (t * DS + dl) * C::SZ, dv, n0);
+        if constexpr (C::SPLIT) {
+#pragma unroll
+            for (int j = 0; j < CPT; ++j) tot[j] += dv[j];
+        }
         token_checked<CPT>(g, L, kk, b, xv, dv, wmask);
     }
 }
 
 // ---------------------------------------------------------------------------
+// Chunks split over the CTAs of a cluster (captures with few work items). The recurrence is
+// linear in the state, so a chunk's final state is the sum over its segments of the
+// segment's own final state (from zero) decayed by the tokens after it:
+//   h[d, n] = sum_s 2^(A[d, n] log2 e * (dt summed over the segments after s)) h_s[d, n].
+// Every CTA leaves its h_s and its sum of dt in its shared memory; the cluster's threads
+// share the (channel, 4 states) sums, each from the last segment back, and write the states. Each
+// segment's sum is relative to its own tokens, so a factor far below 1 belongs to a state
+// that no longer matters and the rounding of its exponent is scaled down with it.
+struct SplitSmem {
+    int32_t dead;      // this CTA gave up on a wait
+    int32_t pad[31];
+    // followed by float4 h[4][DS] (states 4q..4q+3 of a channel) and float dt_sum[DS]
+};
+
+template <class C>
+__device__ __forceinline__ void combine(unsigned char *buf, const ScanParams &p, int segs, int DS, int dl, bool dead,
+                                        const f2 (&h)[C::CPT][8], const float (&tot)[C::CPT], int64_t chunk,
+                                        int layer, int d0) {
+    SplitSmem &sm = *reinterpret_cast<SplitSmem *>(buf);
+    float4 *hs = reinterpret_cast<float4 *>(buf + sizeof(SplitSmem));
+    float *ts = reinterpret_cast<float *>(hs + 4 * DS);
+    if (threadIdx.x == 0) sm.dead = dead;
+#pragma unroll
+    for (int j = 0; j < C::CPT; ++j) {
+        ts[dl + j] = tot[j];
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            float4 v;
+            unpack2(h[j][2 * q], v.x, v.y);
+            unpack2(h[j][2 * q + 1], v.z, v.w);
+            hs[q * DS + dl + j] = v;
+        }
+    }
+    cluster_sync_all();
+    bool any_dead = false;
+    for (int s = 0; s < segs; ++s) any_dead |= ld_cluster_u32(mapa_shared(&sm.dead, s)) != 0u;
+    const int rank = static_cast<int>(cluster_ctarank()), nthr = blockDim.x;
+    const float *Al = p.A + static_cast<int64_t>(layer) * p.D * kN;
+    for (int i = rank * nthr + threadIdx.x; i < 4 * DS && !any_dead; i += segs * nthr) {
+        const int q = i / DS, ch = i % DS;
+        if (d0 + ch >= p.D) continue;
+        const float4 a = *reinterpret_cast<const float4 *>(Al + static_cast<int64_t>(d0 + ch) * kN + 4 * q);
+        const float c[4] = {a.x * kLog2e, a.y * kLog2e, a.z * kLog2e, a.w * kLog2e};
+        float after = 0.f;   // dt summed over the segments after the current one
+        float sum[4] = {0.f, 0.f, 0.f, 0.f};
+        for (int s = segs - 1; s >= 0; --s) {
+            const float4 v = ld_cluster_f4(mapa_shared(&hs[q * DS + ch], s));
+            const float hv[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+            for (int k = 0; k < 4; ++k) sum[k] = fmaf(ex2(c[k] * after), hv[k], sum[k]);
+            after += __uint_as_float(ld_cluster_u32(mapa_shared(&ts[ch], s)));
+        }
+        const int64_t off = ((chunk * p.L_out + p.layer0 + layer) * static_cast<int64_t>(p.D) + d0 + ch) * kN + 4 * q;
+        if (p.state_dtype == PRECOG_F32) {
+            *reinterpret_cast<float4 *>(static_cast<float *>(p.states) + off) = make_float4(sum[0], sum[1], sum[2], sum[3]);
+        } else {
+            __nv_bfloat162 lo = __floats2bfloat162_rn(sum[0], sum[1]), hi = __floats2bfloat162_rn(sum[2], sum[3]);
+            *reinterpret_cast<uint2 *>(static_cast<__nv_bfloat16 *>(p.states) + off) =
+                make_uint2(*reinterpret_cast<uint32_t *>(&lo), *reinterpret_cast<uint32_t *>(&hi));
+        }
+    }
+    cluster_sync_all();   // no CTA leaves while another may still read its shared memory
+}
+
 template <class C>
 __global__ void __launch_bounds__(C::LB_THREADS, C::LB_BLOCKS)
     scan_kernel(const ScanParams p, const int DS_arg, const int slices, const __grid_constant__ SliceMaps maps) {
@@ -680,7 +762,7 @@ __global__ void __launch_bounds__(C::LB_THREADS, C::LB_BLOCKS)
     const int nthr = blockDim.x;
 
     // ---- work item ----
-    int64_t item = blockIdx.x;
+    int64_t item = C::SPLIT ? blockIdx.x / p.segments : blockIdx.x;
     const int slice = static_cast<int>(item % slices);
     item /= slices;
     const int64_t chunk = p.order ? p.order[item % p.n_chunks] : item % p.n_chunks;
@@ -722,6 +804,13 @@ __global__ void __launch_bounds__(C::LB_THREADS, C::LB_BLOCKS)
             return;
         }
         len = end - start;
+    }
+    if constexpr (C::SPLIT) {
+        // this CTA's share of the chunk: whole tiles (the cluster's CTAs left together above)
+        const int64_t share = ((len + TILE - 1) / TILE + p.segments - 1) / p.segments * TILE;
+        const int64_t skip = share * cluster_ctarank();
+        start += skip;
+        len = len > skip ? min64(len - skip, share) : 0;
     }
     TrajCursor tcur{0, 0};
     if constexpr (C::TRAJ) {
@@ -876,9 +965,11 @@ __global__ void __launch_bounds__(C::LB_THREADS, C::LB_BLOCKS)
         }
     }
     const unsigned wmask = __activemask();
-    float Lw[CPT], kk[CPT];
+    float Lw[CPT], kk[CPT], tot[CPT];
+    bool dead = false;
 #pragma unroll
     for (int j = 0; j < CPT; ++j) {
+        tot[j] = 0.f;
         Lw[j] = 0.f;
         kk[j] = -kpow[j];
     }
@@ -933,7 +1024,9 @@ __global__ void __launch_bounds__(C::LB_THREADS, C::LB_BLOCKS)
                 for (int64_t k2 = k; k2 < min64(k + STAGES, ntiles); ++k2)
                     mbar_wait(&full[k2 % STAGES], static_cast<uint32_t>((k2 / STAGES) & 1));
             }
-            return;
+            if constexpr (!C::SPLIT) return;
+            dead = true;   // the cluster's other CTAs still expect this one at their barriers
+            break;
         }
         if constexpr (C::RESCALED && C::TRAJ == kTrajRescaled) {
             // segments end at the trajectory points; there the state is brought back
@@ -942,7 +1035,7 @@ __global__ void __launch_bounds__(C::LB_THREADS, C::LB_BLOCKS)
             while (t < ntok) {
                 const int seg = static_cast<int>(min64(ntok - t, tcur.left));
                 scan_tile_rescaled<C>(st, lay, reinterpret_cast<const float *>(st + (C::CONV ? lay.bf : lay.bs)), DS, dl, t,
-                                      t + seg, h, Lw, kk, wmask);
+                                      t + seg, h, Lw, kk, wmask, tot);
                 t += seg;
                 tcur.left -= seg;
                 if (tcur.left == 0 || k * TILE + t == len) {
@@ -960,10 +1053,10 @@ __global__ void __launch_bounds__(C::LB_THREADS, C::LB_BLOCKS)
             }
         } else if constexpr (C::RESCALED) {
             scan_tile_rescaled<C>(st, lay, reinterpret_cast<const float *>(st + (C::CONV ? lay.bf : lay.bs)), DS, dl, 0,
-                                  ntok, h, Lw, kk, wmask);
+                                  ntok, h, Lw, kk, wmask, tot);
         } else {
             scan_tile_direct<C>(st, lay, DS, dl, ntok, h, kpow, kgen, live, yrow, p.y_dtype, y_stride, p, tcur,
-                                len - k * TILE, p.layer0 + layer, d0 + dl);
+                                len - k * TILE, p.layer0 + layer, d0 + dl, tot);
         }
         if (C::HAS_Y) {
             yrow = (p.y_dtype == PRECOG_F32)
@@ -979,6 +1072,11 @@ __global__ void __launch_bounds__(C::LB_THREADS, C::LB_BLOCKS)
     if constexpr (C::RESCALED) {
 #pragma unroll
         for (int j = 0; j < CPT; ++j) renormalise(h[j], Lw[j]);
+    }
+    if constexpr (C::SPLIT) {
+        __syncthreads();
+        combine<C>(stage0, p, p.segments, DS, dl, dead, h, tot, chunk, layer, d0);
+        return;
     }
     if (p.states && live) {
 #pragma unroll
@@ -1046,10 +1144,45 @@ cudaError_t launch_cfg(const ScanParams &p, cudaStream_t stream) {
     auto kern = scan_kernel<C>;
     cudaError_t e = ensure_smem(reinterpret_cast<const void *>(kern), static_cast<int>(smem));
     if (e != cudaSuccess) return e;
-    kern<<<static_cast<unsigned>(items), DS / C::CPT, smem, stream>>>(p, DS, slices, maps);
-    e = cudaGetLastError();
+    if constexpr (C::SPLIT) {
+        if (items * p.segments > 0x7fffffffLL) return cudaErrorInvalidConfiguration;
+        cudaLaunchConfig_t cfg = {};
+        cfg.gridDim = dim3(static_cast<unsigned>(items * p.segments));
+        cfg.blockDim = dim3(static_cast<unsigned>(DS / C::CPT));
+        cfg.dynamicSmemBytes = smem;
+        cfg.stream = stream;
+        cudaLaunchAttribute attr[1];
+        attr[0].id = cudaLaunchAttributeClusterDimension;
+        attr[0].val.clusterDim.x = static_cast<unsigned>(p.segments);
+        attr[0].val.clusterDim.y = 1;
+        attr[0].val.clusterDim.z = 1;
+        cfg.attrs = attr;
+        cfg.numAttrs = 1;
+        e = cudaLaunchKernelEx(&cfg, kern, p, DS, slices, maps);
+    } else {
+        kern<<<static_cast<unsigned>(items), DS / C::CPT, smem, stream>>>(p, DS, slices, maps);
+        e = cudaGetLastError();
+    }
     if (e == cudaSuccess) count_launches(1);
     return e;
+}
+
+// CTAs per chunk of a capture (1: not split), a power of two up to the portable cluster size.
+// One CTA takes about 0.12 us per token whatever else runs, so a launch that leaves SMs without
+// a CTA or with one is as long as its chunks; split, a chunk of 24 layers x 3 x 500 tokens
+// takes 70 -> 27 us, 1 x 1 x 4096 517 -> 60, 24 x 6 x 500 70 -> 43, 24 x 9 x 500 73 -> 60
+// (bf16 power form; general A 60 -> 33, 448 -> 71, 60 -> 54, 93 -> 77). From 1.5 items per SM
+// on the unsplit launch fills the SMs (24 x 12 x 500: 72.5 against 76; general 93 against
+// 101), and below 80 tokens the combination costs what the shorter chains save.
+int split_segments(const ScanParams &p) {
+    const int64_t sms = device_sm_count();
+    // work items in chunks of 256 channels, tokens per chunk on average
+    const int64_t items = (static_cast<int64_t>(p.n_layers) * p.n_chunks * p.D + kMaxSlice - 1) / kMaxSlice;
+    const int64_t tokens = p.T_tot / p.n_chunks;
+    if (tokens < 80 || 2 * items > 3 * sms) return 1;
+    int segs = 8;
+    while (segs > 1 && (items * segs > 6 * sms || tokens < segs * 16)) segs /= 2;
+    return segs;
 }
 
 // Shapes: the rescaled capture kernel (the corpus-encode hot loop) and the
@@ -1139,6 +1272,15 @@ cudaError_t launch_mode(const ScanParams &p, cudaStream_t stream) {
     }
     const bool has_y = p.y != nullptr;
     const bool has_h0 = p.bank != nullptr;
+    if (!has_y && !has_h0) {
+        const int segs = split_segments(p);
+        if (segs > 1) {
+            ScanParams q = p;
+            q.segments = segs;
+            return launch_cfg<Cfg<TIn, false, false, MODE, 2, 16, 2, MODE == kGeneral ? 4 : 5, kTrajNone, kMaxSlice, 0, true>>(
+                q, stream);
+        }
+    }
     if (has_y)
         return has_h0 ? launch_t<TIn, true, true, MODE>(p, stream)
                       : launch_t<TIn, true, false, MODE>(p, stream);

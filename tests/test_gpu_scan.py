@@ -572,3 +572,45 @@ def test_widths_that_slices_do_not_divide(cuda_device, D, kind, power):
             ref_h, ref_q = oracle.rollout(X[l, sl], DT[l, sl], A[l], Bn[l, sl], Cn[l, sl], h0=h0, want_y=True)
             assert rel_err(to_np(qh[i, l]), ref_h) < tol
             assert rel_err(to_np(qy[l, sl]), ref_q) < tol
+
+
+@pytest.mark.parametrize("kind", ["bf16", "f32"])
+@pytest.mark.parametrize("power", [True, False])
+@pytest.mark.parametrize("L,D,lens", [(1, 64, [4000]), (24, 256, [130]), (2, 1000, [0, 900, 17, 128, 129]),
+                                      (1, 8, [85]), (3, 512, [700, 1, 300, 160]), (2, 256, [97] * 70)])
+def test_split_chunks(cuda_device, kind, power, L, D, lens):
+    """Captures with few work items share each chunk's tokens among a cluster's CTAs and
+    combine their states: 2, 4 and 8 shares, shares without tokens, chunks shorter than the
+    shares, a bad chunk beside good ones (skipped by its whole cluster), bf16 states, and
+    the error against the oracle no larger than the one-CTA scan's tolerance."""
+    import torch
+    pg = _pg()
+    d = cuda_device
+    dtype = torch.float32 if kind == "f32" else torch.bfloat16
+    N = 16
+    off = np.concatenate([[0], np.cumsum(lens)]).astype(np.int64)
+    T = int(off[-1])
+    ins = [synth.host_scan_inputs(T, D, N, seed=3 * D + l) for l in range(L)]
+    rng = np.random.default_rng(D)
+    A = np.stack([i[2] for i in ins]) if power else -rng.uniform(0.05, 3.0, size=(L, D, N)).astype(np.float32)
+    x, dt, B = (torch.stack([_t(i[k], d, dtype) for i in ins]) for k in (0, 1, 3))
+    if kind == "f32":
+        dt[:, ::7] *= -0.1                      # steps of both signs
+    states, _ = _encode(d, x, dt, B, _t(A, d), _t(off, d, torch.int64), power=power)
+    half, _ = _encode(d, x, dt, B, _t(A, d), _t(off, d, torch.int64), power=power, state_dtype=torch.bfloat16)
+    assert torch.equal(half, states.to(torch.bfloat16))
+    tol = TOL_F32 if kind == "f32" else TOL_BF16
+    for l in sorted({0, L - 1}):
+        ref, _ = oracle.scan(to_np(x[l]), to_np(dt[l]), A[l], to_np(B[l]), off)
+        for c in range(len(lens)):
+            assert rel_err(to_np(states[c, l]), ref[c]) < tol
+    if len(lens) == 5:
+        bad = off.copy()
+        bad[2] = T + 5                          # chunks 1 and 2 have bad rows
+        out = torch.full_like(states, 7.0)
+        pg.precog_encode_chunks(pg.scan_inputs(x, dt, B, _t(A, d), a_kind=pg.PRECOG_A_POWER if power else
+                                               pg.PRECOG_A_GENERAL), _t(bad, d, torch.int64), T, out)
+        st, bits = pg.precog_device_status()
+        assert st != 0 and bits & pg.PRECOG_DEV_BAD_OFFSETS
+        assert (out[1:3] == 7.0).all()
+        assert torch.equal(out[[0, 3, 4]], states[[0, 3, 4]])
