@@ -85,6 +85,9 @@ struct Cfg {
     static constexpr int FIXDS = FIXDS_;
     // A cluster of CTAs per work item, each with a share of the chunk's tokens (see combine).
     static constexpr bool SPLIT = SPLIT_;
+    // 256-channel slices that stand in for 512-channel ones: the power statement is verified
+    // for the 512 channels together, as by those.
+    static constexpr bool WIDE_CHECK = MODE_ == kPower && CPT_ == 2 && (SPLIT_ || MINB_ == 4);
     // Widest channel slice of one CTA. Each CTA stages its slice of every token row; a
     // slice narrower than the row turns the row into separate pieces, and HBM serves
     // short scattered pieces far below its streaming rate, so rows up to 512 channels
@@ -848,6 +851,23 @@ __global__ void __launch_bounds__(C::LB_THREADS, C::LB_BLOCKS)
             for (int n = 1; n < kN; ++n) a_ok &= a[n] == static_cast<float>(n + 1) * a[0];
         }
     }
+    if constexpr (C::WIDE_CHECK) {
+        if (DS == kMaxSlice && D % kWideSlice == 0) {
+            const float4 *a4 = reinterpret_cast<const float4 *>(
+                p.A + (static_cast<int64_t>(layer) * D + (slice ^ 1) * DS + dl) * kN);
+#pragma unroll
+            for (int j = 0; j < CPT; ++j) {
+                const float a0 = a4[j * (kN / 4)].x;
+                a_ok &= a0 <= 0.f;
+#pragma unroll
+                for (int q = 0; q < kN / 4; ++q) {
+                    const float4 v = a4[j * (kN / 4) + q];
+                    const float n = static_cast<float>(4 * q + 1);
+                    a_ok &= v.x == n * a0 && v.y == (n + 1.f) * a0 && v.z == (n + 2.f) * a0 && v.w == (n + 3.f) * a0;
+                }
+            }
+        }
+    }
     if constexpr (C::MODE == kPower) {
         if (!__syncthreads_and(a_ok)) {
             if (tid == 0) atomicOr(&g_scan_status, PRECOG_DEV_BAD_A);
@@ -1185,6 +1205,19 @@ int split_segments(const ScanParams &p) {
     return segs;
 }
 
+// Two channels per thread, 128 registers, four CTAs of 256 channels per SM: power-form A with
+// fp32 inputs. Their tiles are twice as large, so that with four channels per thread three CTAs
+// of two warps were left to an SM; this shape has 16 warps: 1 layer x 500 chunks x 1000 tokens
+// capture 274 -> 231 us, 1 x 100 x 300 x 2048 144 -> 112; readout 24 x 30 x 500 370 -> 290,
+// 1 x 100 x 300 x 2048 276 -> 215. (bf16 captures of this shape take 215 -> 234 us, readouts
+// 190 -> 209.)
+template <typename TIn, bool HAS_Y, bool HAS_H0, int TRAJ>
+cudaError_t launch_pairs(const ScanParams &p, cudaStream_t stream) {
+    if (p.D % kMaxSlice == 0)
+        return launch_cfg<Cfg<TIn, HAS_Y, HAS_H0, kPower, 2, 16, 2, 4, TRAJ, kMaxSlice, kMaxSlice>>(p, stream);
+    return launch_cfg<Cfg<TIn, HAS_Y, HAS_H0, kPower, 2, 16, 2, 4, TRAJ, kMaxSlice>>(p, stream);
+}
+
 // Shapes: the rescaled capture kernel (the corpus-encode hot loop) and the
 // direct kernels (readout, prefill, general A).
 template <typename TIn, bool HAS_Y, bool HAS_H0, int MODE, int TRAJ = kTrajNone>
@@ -1209,7 +1242,8 @@ cudaError_t launch_t(const ScanParams &p, cudaStream_t stream) {
     } else if constexpr (MODE == kPower && !HAS_Y) {
         // the corpus encode of 256- and 512-channel slices (the paper's layer width, the
         // ragged and wide workloads' slices) gets the slice fixed at compile time
-        if constexpr (!HAS_H0 && !std::is_same<TIn, float>::value) {
+        if constexpr (std::is_same<TIn, float>::value) return launch_pairs<TIn, HAS_Y, HAS_H0, kTrajNone>(p, stream);
+        if constexpr (!HAS_H0) {
             const int ds = pick_slice(p.D, kWideSlice);
             if (ds == 256 && p.D % 256 == 0)
                 return launch_cfg<Cfg<TIn, false, false, MODE, PRECOG_RESCALED_CPT, PRECOG_RESCALED_TILE,
@@ -1231,18 +1265,15 @@ cudaError_t launch_t(const ScanParams &p, cudaStream_t stream) {
                 if (scan_latency_eligible(p)) return launch_scan_latency(p, stream);
                 return launch_cfg<Cfg<TIn, HAS_Y, HAS_H0, MODE, 2, 16, 2, 3>>(p, stream);
             }
-            if constexpr (!std::is_same<TIn, float>::value) {
-                // 16-bit rows: 256- and 512-channel slices fixed at compile time
-                const int ds = pick_slice(p.D, kWideSlice);
-                if (ds == 256 && p.D % 256 == 0)
-                    return launch_cfg<Cfg<TIn, HAS_Y, HAS_H0, MODE, PRECOG_DIRECT_CPT, PRECOG_DIRECT_TILE,
-                                          PRECOG_DIRECT_STAGES, PRECOG_DIRECT_MINB, kTrajNone, kWideSlice, 256>>(
-                        p, stream);
-                if (ds == 512)
-                    return launch_cfg<Cfg<TIn, HAS_Y, HAS_H0, MODE, PRECOG_DIRECT_CPT, PRECOG_DIRECT_TILE,
-                                          PRECOG_DIRECT_STAGES, PRECOG_DIRECT_MINB, kTrajNone, kWideSlice, 512>>(
-                        p, stream);
-            }
+            if constexpr (std::is_same<TIn, float>::value) return launch_pairs<TIn, HAS_Y, HAS_H0, kTrajNone>(p, stream);
+            // 16-bit rows: 256- and 512-channel slices fixed at compile time
+            const int ds = pick_slice(p.D, kWideSlice);
+            if (ds == 256 && p.D % 256 == 0)
+                return launch_cfg<Cfg<TIn, HAS_Y, HAS_H0, MODE, PRECOG_DIRECT_CPT, PRECOG_DIRECT_TILE,
+                                      PRECOG_DIRECT_STAGES, PRECOG_DIRECT_MINB, kTrajNone, kWideSlice, 256>>(p, stream);
+            if (ds == 512)
+                return launch_cfg<Cfg<TIn, HAS_Y, HAS_H0, MODE, PRECOG_DIRECT_CPT, PRECOG_DIRECT_TILE,
+                                      PRECOG_DIRECT_STAGES, PRECOG_DIRECT_MINB, kTrajNone, kWideSlice, 512>>(p, stream);
             return launch_cfg<Cfg<TIn, HAS_Y, HAS_H0, MODE, PRECOG_DIRECT_CPT, PRECOG_DIRECT_TILE,
                                   PRECOG_DIRECT_STAGES, PRECOG_DIRECT_MINB, kTrajNone, kWideSlice>>(p, stream);
         } else {

@@ -604,6 +604,15 @@ def test_split_chunks(cuda_device, kind, power, L, D, lens):
         ref, _ = oracle.scan(to_np(x[l]), to_np(dt[l]), A[l], to_np(B[l]), off)
         for c in range(len(lens)):
             assert rel_err(to_np(states[c, l]), ref[c]) < tol
+    if power and D == 512:
+        Ab = A.copy()
+        Ab[1, 300, 5] *= 1.5                    # the statement is verified for 512 channels together
+        out = torch.full_like(states, 7.0)
+        pg.precog_encode_chunks(pg.scan_inputs(x, dt, B, _t(Ab, d), a_kind=pg.PRECOG_A_POWER),
+                                _t(off, d, torch.int64), T, out)
+        st, bits = pg.precog_device_status()
+        assert st != 0 and bits == pg.PRECOG_DEV_BAD_A
+        assert (out[:, 1] == 7.0).all() and torch.equal(out[:, 0], states[:, 0])
     if len(lens) == 5:
         bad = off.copy()
         bad[2] = T + 5                          # chunks 1 and 2 have bad rows
