@@ -62,6 +62,13 @@ __device__ uint32_t g_scan_status;
 #endif
 
 
+// Tokens whose exponentials the direct update forms ahead: their latency and the loads' then
+// overlap the previous tokens' chains. Against one token at a time: readout of 256 chunks x 512
+// tokens x 2048 channels 689 -> 652 us, 4 layers x 1000 x 500 1307 -> 1218; trajectories (every
+// 8th state of 4 x 128 x 750) 414 -> 340; groups of 2: 670, 1268, 348; of 8: 3 % slower than 4
+// in the readouts; of a whole tile 50 % (registers).
+constexpr int kDirectGroup = 4;
+
 constexpr int kN = 16;          // state size (N) supported by the kernels
 constexpr int kMaxSlice = 256;  // channels per CTA at most (the default slice)
 constexpr int kWideSlice = 512; // rows of up to this many channels are staged whole
@@ -344,49 +351,57 @@ __device__ __forceinline__ void scan_tile_direct(const unsigned char *st, const 
     constexpr int CPT = C::CPT;
     const float *bsrc = reinterpret_cast<const float *>(st + (C::CONV ? lay.bf : lay.bs));
     const float *csrc = reinterpret_cast<const float *>(st + (C::CONV ? lay.cf : lay.cs));
-    for (int t = 0; t < ntok; ++t) {
+    // dt and x of a token: raw words of 16-bit inputs (u = dt * x is formed from the halves,
+    // exactly, and x never widened), else values
+    struct Chan {
+        uint32_t xw[CPT / 2], dw[CPT / 2];
+        float xv[CPT], dv[CPT], r[CPT];
+    };
+    auto fetch = [&](int t, Chan &c) {
+        if constexpr (C::CONV) {
+            load_words<CPT>(st + lay.xs + (t * DS + dl) * C::SZ, c.xw);
+            load_words<CPT>(st + lay.dts + (t * DS + dl) * C::SZ, c.dw);
+            widen_words<CPT>(c.dw, c.dv);
+        } else {
+            uint32_t neg;
+            load_chan<typename C::TIn, CPT>(st + lay.xs + (t * DS + dl) * C::SZ, c.xv, neg);
+            load_chan<typename C::TIn, CPT>(st + lay.dts + (t * DS + dl) * C::SZ, c.dv, neg);
+        }
+        if constexpr (C::MODE == kPower) {
+#pragma unroll
+            for (int j = 0; j < CPT; ++j) c.r[j] = ex2(c.dv[j] * kpow[j]);
+        }
+    };
+    auto token = [&](int t, const Chan &c) {
         f2 b[8];
         load_b(bsrc, t, b);
-        float xv[CPT], dv[CPT], yv[CPT] = {}, uv[CPT];
-        uint32_t neg;
-        f2 uu2[CPT];   // (u, u) pairs of the 16-bit path, both halves computed
+        float yv[CPT] = {};
+        f2 uu2[CPT];   // (u, u)
         if constexpr (C::CONV) {
-            // u = dt * x from the raw bf16 halves (exact), x never widened
-            uint32_t xw[CPT / 2], dw[CPT / 2];
-            load_words<CPT>(st + lay.xs + (t * DS + dl) * C::SZ, xw);
-            load_words<CPT>(st + lay.dts + (t * DS + dl) * C::SZ, dw);
-            widen_words<CPT>(dw, dv);
+            // both halves computed: two products cost less than a product and a move
 #pragma unroll
             for (int i = 0; i < CPT / 2; ++i) {
-                uv[2 * i] = mul_bf16_lo(dw[i], xw[i]);
-                uv[2 * i + 1] = mul_bf16_hi(dw[i], xw[i]);
-            }
-#pragma unroll
-            for (int i = 0; i < CPT / 2; ++i) {
-                uu2[2 * i] = pack2(mul_bf16_lo_v(dw[i], xw[i]), mul_bf16_lo_v(dw[i], xw[i]));
-                uu2[2 * i + 1] = pack2(mul_bf16_hi_v(dw[i], xw[i]), mul_bf16_hi_v(dw[i], xw[i]));
+                uu2[2 * i] = pack2(mul_bf16_lo_v(c.dw[i], c.xw[i]), mul_bf16_lo_v(c.dw[i], c.xw[i]));
+                uu2[2 * i + 1] = pack2(mul_bf16_hi_v(c.dw[i], c.xw[i]), mul_bf16_hi_v(c.dw[i], c.xw[i]));
             }
         } else {
-            load_chan<typename C::TIn, CPT>(st + lay.xs + (t * DS + dl) * C::SZ, xv, neg);
-            load_chan<typename C::TIn, CPT>(st + lay.dts + (t * DS + dl) * C::SZ, dv, neg);
 #pragma unroll
-            for (int j = 0; j < CPT; ++j) uv[j] = dv[j] * xv[j];
+            for (int j = 0; j < CPT; ++j) uu2[j] = pack2(c.dv[j] * c.xv[j], c.dv[j] * c.xv[j]);
         }
         if constexpr (C::SPLIT) {
 #pragma unroll
-            for (int j = 0; j < CPT; ++j) tot[j] += dv[j];
+            for (int j = 0; j < CPT; ++j) tot[j] += c.dv[j];
         }
 #pragma unroll
         for (int j = 0; j < CPT; ++j) {
-            const float u = uv[j];
-            const f2 uu = C::CONV ? uu2[j] : pack2(u, u);
+            const f2 uu = uu2[j];
             if constexpr (C::MODE == kPower) {
                 f2 a[8];
-                pow_pairs_direct(ex2(dv[j] * kpow[j]), a);
+                pow_pairs_direct(c.r[j], a);
 #pragma unroll
                 for (int i = 0; i < 8; ++i) h[j][i] = fma2(a[i], h[j][i], mul2(uu, b[i]));
             } else {
-                const f2 dd = pack2(dv[j], dv[j]);
+                const f2 dd = pack2(c.dv[j], c.dv[j]);
 #pragma unroll
                 for (int i = 0; i < 8; ++i) {
                     float e0, e1;
@@ -441,6 +456,22 @@ __device__ __forceinline__ void scan_tile_direct(const unsigned char *st, const 
                 tc.left = p.traj_stride;
             }
         }
+    };
+    constexpr int G = C::MODE == kPower ? kDirectGroup : 1;   // general A: 16 exponentials per token already
+    int t = 0;
+    if constexpr (G > 1) {
+        for (; t + G <= ntok; t += G) {
+            Chan c[G];
+#pragma unroll
+            for (int g = 0; g < G; ++g) fetch(t + g, c[g]);
+#pragma unroll
+            for (int g = 0; g < G; ++g) token(t + g, c[g]);
+        }
+    }
+    for (; t < ntok; ++t) {
+        Chan c;
+        fetch(t, c);
+        token(t, c);
     }
 }
 
