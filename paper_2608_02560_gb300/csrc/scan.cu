@@ -108,6 +108,8 @@ struct Cfg {
     // keep every stride-th state (K-dial, Sec. 5.2), with the direct or the rescaled update
     static constexpr int TRAJ = TRAJ_;
     static constexpr int MODE = MODE_, CPT = CPT_, TILE = TILE_, STAGES = STAGES_;
+    // trajectory states leave through shared memory (see store_trajectory)
+    static constexpr bool STAGED = TRAJ_ != kTrajNone && MODE_ == kPower && CPT_ == 2;
     static constexpr bool CONV = !std::is_same<TIn_, float>::value;
     static constexpr int SZ = sizeof(TIn_);
     static constexpr bool RESCALED = MODE_ == kPower && !HAS_Y_ && TRAJ_ != kTrajDirect;
@@ -117,6 +119,9 @@ struct Cfg {
 struct TrajCursor {
     int64_t entry;
     int64_t left;
+    // the warp's staging buffers, which of them is next, and its channels
+    unsigned char *bufs;
+    int which, channels, first;
 };
 
 // Tensor maps of x and dt for launches whose CTAs take a slice of each row: the tensor is
@@ -338,6 +343,80 @@ __device__ __forceinline__ void widen_words(const uint32_t (&w)[CPT / 2], float 
 }
 
 // ---------------------------------------------------------------------------
+// Trajectory states. The states of a warp's channels are adjacent in an entry, but a thread's
+// are 32 to 128 bytes apart from its neighbour's, so plain stores of 16 bytes touched 32 lines
+// each with half a sector and bound the fine strides. A warp instead lays its states out in a
+// shared-memory buffer (rotating the 16-byte pieces by lane, so that the lanes meet different
+// banks) and one lane sends them off as a bulk copy; a warp has two buffers of bf16 states or
+// one of fp32. With two channels per thread (launch_pairs), 4 layers x 40 chunks x 750 tokens,
+// every state bf16 615 -> 476 us and fp32 1253 -> 565, every third (100 chunks) 472 -> 386 and
+// 801 -> 538; strides 16 to 100 5 to 25 % (435, 457, 329, 520 with the grouped direct update).
+__host__ __device__ constexpr int traj_buffer_bytes(int cpt) { return 2 * 32 * cpt * kN * 2; }   // per warp
+
+template <int CPT>
+__device__ __forceinline__ void store_trajectory(unsigned char *bufs, int &which, int lane, int channels, void *base,
+                                                 int dtype, int64_t elem_off, const f2 (&h)[CPT][8]) {
+    if (channels <= 0) return;   // a warp past the end of the row (uniform)
+    // the copy before the last one (fp32: the last one) has left the buffer
+    if (lane == 0) {
+        if (dtype == PRECOG_F32) bulk_wait_read<0>();
+        else bulk_wait_read<1>();
+    }
+    __syncwarp();
+    unsigned char *buf = dtype == PRECOG_F32 ? bufs : bufs + which * (traj_buffer_bytes(CPT) / 2);
+    which ^= 1;
+    const int rot = (lane >> 1) & 3;
+    // blocks of four 16-byte pieces: half a channel's fp32 states twice over, or two channels' bf16
+    auto put = [&](int block, int blocks, const uint4 (&p)[4]) {
+        uint4 r[4], q[4];
+#pragma unroll
+        for (int i = 0; i < 4; ++i) r[i] = rot & 1 ? p[(i + 1) & 3] : p[i];
+#pragma unroll
+        for (int i = 0; i < 4; ++i) q[i] = rot & 2 ? r[(i + 2) & 3] : r[i];
+        uint4 *dst = reinterpret_cast<uint4 *>(buf) + (lane * blocks + block) * 4;
+#pragma unroll
+        for (int i = 0; i < 4; ++i) dst[(i + rot) & 3] = q[i];
+    };
+    static_assert(CPT % 2 == 0, "two channels per block of bf16 pieces");
+    if (dtype == PRECOG_F32) {
+#pragma unroll
+        for (int j = 0; j < CPT; ++j) {
+            uint4 p[4];
+#pragma unroll
+            for (int i = 0; i < 4; ++i)
+                p[i] = make_uint4(static_cast<uint32_t>(h[j][2 * i]), static_cast<uint32_t>(h[j][2 * i] >> 32),
+                                  static_cast<uint32_t>(h[j][2 * i + 1]), static_cast<uint32_t>(h[j][2 * i + 1] >> 32));
+            put(j, CPT, p);
+        }
+    } else {
+#pragma unroll
+        for (int j = 0; j < CPT; j += 2) {
+            uint4 p[4];
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                uint32_t w[4];
+#pragma unroll
+                for (int k = 0; k < 4; ++k) {
+                    float lo, hi;
+                    unpack2(h[j + i / 2][(i & 1) * 4 + k], lo, hi);
+                    const __nv_bfloat162 b2 = __floats2bfloat162_rn(lo, hi);
+                    w[k] = *reinterpret_cast<const uint32_t *>(&b2);
+                }
+                p[i] = make_uint4(w[0], w[1], w[2], w[3]);
+            }
+            put(j / 2, CPT / 2, p);
+        }
+    }
+    fence_proxy_async_smem();
+    __syncwarp();
+    if (lane == 0) {
+        const int sz = dtype == PRECOG_F32 ? 4 : 2;
+        bulk_s2g(static_cast<unsigned char *>(base) + elem_off * sz, buf, static_cast<uint32_t>(channels * kN * sz));
+        bulk_commit();
+    }
+}
+
+// ---------------------------------------------------------------------------
 // Direct update (any readout): h_n <- alpha_n h_n + u B_n, y = sum_n C_n h_n.
 template <class C>
 __device__ __forceinline__ void scan_tile_direct(const unsigned char *st, const StageLayout &lay,
@@ -446,12 +525,15 @@ __device__ __forceinline__ void scan_tile_direct(const unsigned char *st, const 
         if constexpr (C::TRAJ == kTrajDirect) {
             // after every stride-th token and after the chunk's last token (uniform)
             if (--tc.left == 0 || t + 1 == tok_left) {
+                const int64_t row = (tc.entry * p.L_out + traj_layer) * static_cast<int64_t>(p.D);
+                if constexpr (C::STAGED) {
+                    store_trajectory<CPT>(tc.bufs, tc.which, threadIdx.x & 31, tc.channels, p.traj, p.traj_dtype,
+                                          (row + tc.first) * kN, h);
+                } else {
 #pragma unroll
-                for (int j = 0; live && j < CPT; ++j)
-                    store_state16(p.traj, p.traj_dtype,
-                                  ((tc.entry * p.L_out + traj_layer) * static_cast<int64_t>(p.D) + dglob + j) *
-                                      kN,
-                                  h[j]);
+                    for (int j = 0; live && j < CPT; ++j)
+                        store_state16(p.traj, p.traj_dtype, (row + dglob + j) * kN, h[j]);
+                }
                 ++tc.entry;
                 tc.left = p.traj_stride;
             }
@@ -846,7 +928,7 @@ __global__ void __launch_bounds__(C::LB_THREADS, C::LB_BLOCKS)
         start += skip;
         len = len > skip ? min64(len - skip, share) : 0;
     }
-    TrajCursor tcur{0, 0};
+    TrajCursor tcur{};
     if constexpr (C::TRAJ) {
         // chunk c keeps ceil(len / stride) states starting at entry traj_offsets[c]
         const int64_t e0 = p.traj_offsets[chunk], e1 = p.traj_offsets[chunk + 1];
@@ -856,6 +938,11 @@ __global__ void __launch_bounds__(C::LB_THREADS, C::LB_BLOCKS)
         }
         tcur.entry = e0;
         tcur.left = p.traj_stride;
+        const int wc = 32 * CPT, w0 = slice * DS + tid / 32 * wc;   // the warp's channels
+        const int row_end = p.D - slice * DS < DS ? p.D : slice * DS + DS;
+        tcur.first = w0;
+        tcur.channels = row_end - w0 < wc ? row_end - w0 : wc;
+        tcur.bufs = stage0 + STAGES * lay.bytes + tid / 32 * traj_buffer_bytes(CPT);
     }
     const int d0 = slice * DS;
     const int dl = tid * CPT;
@@ -1075,6 +1162,9 @@ __global__ void __launch_bounds__(C::LB_THREADS, C::LB_BLOCKS)
                 for (int64_t k2 = k; k2 < min64(k + STAGES, ntiles); ++k2)
                     mbar_wait(&full[k2 % STAGES], static_cast<uint32_t>((k2 / STAGES) & 1));
             }
+            if constexpr (C::STAGED) {
+                if ((tid & 31) == 0) bulk_wait_all();
+            }
             if constexpr (!C::SPLIT) return;
             dead = true;   // the cluster's other CTAs still expect this one at their barriers
             break;
@@ -1091,12 +1181,15 @@ __global__ void __launch_bounds__(C::LB_THREADS, C::LB_BLOCKS)
                 tcur.left -= seg;
                 if (tcur.left == 0 || k * TILE + t == len) {
 #pragma unroll
-                    for (int j = 0; j < CPT; ++j) {
-                        renormalise(h[j], Lw[j]);
-                        if (live) store_state16(p.traj, p.traj_dtype,
-                                      ((tcur.entry * p.L_out + p.layer0 + layer) * static_cast<int64_t>(D) +
-                                       d0 + dl + j) * kN,
-                                      h[j]);
+                    for (int j = 0; j < CPT; ++j) renormalise(h[j], Lw[j]);
+                    const int64_t row = (tcur.entry * p.L_out + p.layer0 + layer) * static_cast<int64_t>(D);
+                    if constexpr (C::STAGED) {
+                        store_trajectory<CPT>(tcur.bufs, tcur.which, tid & 31, tcur.channels, p.traj, p.traj_dtype,
+                                              (row + tcur.first) * kN, h);
+                    } else {
+#pragma unroll
+                        for (int j = 0; live && j < CPT; ++j)
+                            store_state16(p.traj, p.traj_dtype, (row + d0 + dl + j) * kN, h[j]);
                     }
                     ++tcur.entry;
                     tcur.left = p.traj_stride;
@@ -1120,6 +1213,10 @@ __global__ void __launch_bounds__(C::LB_THREADS, C::LB_BLOCKS)
     }
 
     // ---- state capture ----
+    if constexpr (C::STAGED) {
+        if ((tid & 31) == 0) bulk_wait_all();   // the last states are on their way out of shared memory
+        return;
+    }
     if constexpr (C::RESCALED) {
 #pragma unroll
         for (int j = 0; j < CPT; ++j) renormalise(h[j], Lw[j]);
@@ -1163,13 +1260,20 @@ bool few_channels(const ScanParams &p) {
     return static_cast<int64_t>(p.n_layers) * p.n_chunks * p.D < static_cast<int64_t>(device_sm_count()) * kMaxSlice;
 }
 
+// At least six chunks of 256 channels per SM.
+bool many_channels(const ScanParams &p) {
+    return static_cast<int64_t>(p.n_layers) * p.n_chunks * p.D >= 6 * static_cast<int64_t>(device_sm_count()) * kMaxSlice;
+}
+
 template <class C>
 cudaError_t launch_cfg(const ScanParams &p, cudaStream_t stream) {
     const int DS = C::FIXDS ? C::FIXDS : pick_slice(p.D, C::MAXSLICE);
     if (DS % C::CPT != 0 || (C::FIXDS && p.D % DS != 0)) return cudaErrorInvalidValue;
     const int slices = (p.D + DS - 1) / DS;
     const StageLayout lay = stage_layout(C::TILE, DS, C::SZ, C::HAS_Y, C::CONV);
-    const size_t smem = kBarBytes + static_cast<size_t>(C::STAGES) * lay.bytes;
+    const int warps = (DS / C::CPT + 31) / 32;
+    const size_t smem = kBarBytes + static_cast<size_t>(C::STAGES) * lay.bytes +
+                        (C::STAGED ? warps * traj_buffer_bytes(C::CPT) : 0);
     const int64_t items = static_cast<int64_t>(p.n_layers) * p.n_chunks * slices;
     if (items == 0) return cudaSuccess;
     if (items > 0x7fffffffLL) return cudaErrorInvalidConfiguration;
@@ -1253,21 +1357,23 @@ cudaError_t launch_pairs(const ScanParams &p, cudaStream_t stream) {
 // direct kernels (readout, prefill, general A).
 template <typename TIn, bool HAS_Y, bool HAS_H0, int MODE, int TRAJ = kTrajNone>
 cudaError_t launch_t(const ScanParams &p, cudaStream_t stream) {
-    if constexpr (TRAJ == kTrajRescaled) {
-        if (p.D % 256 == 0 && p.D % 512 != 0)
-            return launch_cfg<Cfg<TIn, false, false, kPower, PRECOG_RESCALED_CPT, PRECOG_RESCALED_TILE,
-                                  PRECOG_RESCALED_STAGES, PRECOG_RESCALED_MINB, kTrajRescaled, kWideSlice, 256>>(p, stream);
-        return launch_cfg<Cfg<TIn, false, false, kPower, PRECOG_RESCALED_CPT, PRECOG_RESCALED_TILE,
-                              PRECOG_RESCALED_STAGES, PRECOG_RESCALED_MINB, kTrajRescaled, kWideSlice>>(p, stream);
-    } else if constexpr (TRAJ == kTrajDirect) {
-        // short strides and general A: the direct update (h is at hand after every token)
+    if constexpr (TRAJ != kTrajNone) {
+        // power form: the rescaled or (short strides) the direct update, in the fp32 shape for
+        // any input but for wide strides over many 16-bit chunks, which are captures but for a
+        // few stores (stride 1000, 4 x 1000 x 1000 tokens: 1076 us, 1088 in the fp32 shape;
+        // stride 100, 4 x 250 x 750: 374, 345)
         if constexpr (MODE == kPower) {
-            if (p.D % 256 == 0 && p.D % 512 != 0)
-                return launch_cfg<Cfg<TIn, false, false, MODE, PRECOG_DIRECT_CPT, PRECOG_DIRECT_TILE, PRECOG_DIRECT_STAGES,
-                                      PRECOG_DIRECT_MINB, kTrajDirect, kWideSlice, 256>>(p, stream);
-            return launch_cfg<Cfg<TIn, false, false, MODE, PRECOG_DIRECT_CPT, PRECOG_DIRECT_TILE,
-                                  PRECOG_DIRECT_STAGES, PRECOG_DIRECT_MINB, kTrajDirect, kWideSlice>>(p, stream);
+            if constexpr (TRAJ == kTrajRescaled && !std::is_same<TIn, float>::value)
+                if (p.traj_stride >= 256 && many_channels(p))
+                    return p.D % 256 == 0 && p.D % 512 != 0
+                               ? launch_cfg<Cfg<TIn, false, false, kPower, PRECOG_RESCALED_CPT, PRECOG_RESCALED_TILE,
+                                                PRECOG_RESCALED_STAGES, PRECOG_RESCALED_MINB, TRAJ, kWideSlice, 256>>(p, stream)
+                               : launch_cfg<Cfg<TIn, false, false, kPower, PRECOG_RESCALED_CPT, PRECOG_RESCALED_TILE,
+                                                PRECOG_RESCALED_STAGES, PRECOG_RESCALED_MINB, TRAJ, kWideSlice>>(p, stream);
+            return launch_pairs<TIn, false, false, TRAJ>(p, stream);
         } else {
+            if (p.D % 256 == 0)
+                return launch_cfg<Cfg<TIn, false, false, MODE, 2, 16, 4, 3, kTrajDirect, kMaxSlice, 256>>(p, stream);
             return launch_cfg<Cfg<TIn, false, false, MODE, 2, 16, 4, 3, kTrajDirect>>(p, stream);
         }
     } else if constexpr (MODE == kPower && !HAS_Y) {
