@@ -104,7 +104,6 @@ cudaError_t launch_decode_keys(const int64_t *keys, int32_t n, int64_t *best_idx
                                cudaStream_t stream);
 
 // Tensor-core path (retrieve_tc.cu): fp16/bf16 index, batches of queries.
-size_t retrieve_tc_smem_bytes();
 int retrieve_tc_grid(int64_t M, int sms);
 cudaError_t launch_retrieve_tc(const RetrieveParams &p, int grid, cudaStream_t stream,
                                uint64_t *launches);

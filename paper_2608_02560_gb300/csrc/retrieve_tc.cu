@@ -2,10 +2,11 @@
 // cores (Sec. 4.2 query-time retrieval, exact dot product, lowest row on ties).
 //
 // S = Q K^T is a dense contraction once several queries share a pass over the
-// index, so it runs on tcgen05: queries are the A operand, key rows the B operand
-// (tiles of 256 rows), dim the K dimension in blocks of 64 (128 bytes,
-// 128B-swizzled). The query operand is re-read for every key tile, so the key
-// tile is as wide as one MMA allows (N = 256). fp32 accumulators live in tensor
+// index, so it runs on tcgen05: queries are the A operand, key rows the B operand,
+// dim the K dimension in blocks of 64 (128 bytes, 128B-swizzled). The query operand
+// is re-read for every key tile, so the tiles are nearly as tall as one MMA allows
+// (N = 256): the height that spreads the rows evenly over the CTAs' rounds of tiles
+// (tile_rows). fp32 accumulators live in tensor
 // memory; the score matrix never leaves the SM: thread q of the epilogue owns
 // TMEM lane q (one query) and scans its columns (key rows) in increasing order
 // with a strict '>', which keeps the lowest row on ties; NaN never compares
@@ -16,7 +17,8 @@
 // 256 TMEM columns and is double-buffered, so the argmax of one tile overlaps the
 // MMAs of the next; two halves fill all 512 columns with one buffer. Warp roles
 // (320 threads):
-//   warp 0  TMA producer: A (queries) and B (key tile) k-blocks into a 3-stage ring
+//   warp 0  TMA producer: A (queries) and B (key tile) k-blocks into a ring of as many
+//           stages as fit (3 of full tiles, up to kMaxStages of short ones)
 //   warp 1  TMEM owner and MMA issuer (one elected lane)
 //   warps 2-5 / 6-9 epilogue of query half 0 / 1: TMEM -> registers -> running
 //   (score, row) per query
@@ -37,27 +39,42 @@ namespace {
 __device__ uint32_t g_retrieve_status_tc;
 
 constexpr int kBM = 128;          // queries per MMA (one half)
-constexpr int kBN = 256;          // key rows per tile
+constexpr int kBN = 256;          // key rows per tile at most (a multiple of 32)
 constexpr int kBK = 64;           // dim per k-block (128 bytes of fp16/bf16)
-constexpr int kStages = 3;
+constexpr int kMinRows = 64;      // and at least
+// Keys in flight per CTA: more of them queue in the memory system (192 KB: 1M x 768 keys 220
+// instead of 215 us; 128 KB of full tiles: 1M x 1024 286 instead of 284), less starve short tiles.
+constexpr uint32_t kKeyBytes = 112 * 1024;
+constexpr int kMaxStages = kKeyBytes / (kMinRows * kBK * 2);
 constexpr int kTopkStride = 8;    // keys per (CTA, query) in the top-k workspace
 constexpr int kThreads = 320;     // 2 control warps + 8 epilogue warps
 constexpr uint32_t kTmemCols = 512;
-constexpr uint32_t kABytes = kBM * kBK * 2;   // one query half per stage
-constexpr uint32_t kBBytes = kBN * kBK * 2;
+constexpr uint32_t kRowBytes = kBK * 2;       // bytes of a row in a k-block
+constexpr uint32_t kABytes = kBM * kRowBytes;   // one query half per stage
+constexpr int kFewQueries = 32;   // up to here an A tile has 32 rows: the MMA's other rows read
+                                  // whatever follows them, and their lanes are never read back
+constexpr uint32_t kRingBytes = 3 * (2 * kABytes + kBN * kRowBytes);   // 192 KB
 
 struct Smem {
-    // 1024-byte aligned operand tiles (128B swizzle atoms are 8 rows x 128 B)
-    uint8_t a[kStages][2][kABytes];
-    uint8_t b[kStages][kBBytes];
-    uint64_t full[kStages];
-    uint64_t empty[kStages];
+    // stages of [query halves][key rows], 1024-byte aligned operand tiles (128B swizzle atoms
+    // are 8 rows x 128 B). What follows the ring also covers the last A tile's stray reads.
+    uint8_t ring[kRingBytes];
+    uint64_t full[kMaxStages];
+    uint64_t empty[kMaxStages];
     uint64_t acc_full[2];
     uint64_t acc_empty[2];
     uint32_t tmem_base;
     uint32_t abort_flag;
     // epilogue scratch: one row of 32 scores per epilogue thread (padded: conflict-free)
     float epi[8 * 32][33];
+};
+static_assert(sizeof(Smem) - kRingBytes >= kABytes, "stray A reads stay inside the CTA's shared memory");
+
+// The ring's shape for one launch.
+struct Ring {
+    int bn;             // key rows per tile
+    int stages;
+    uint32_t a_bytes;   // of one query half
 };
 
 // Shared-memory matrix descriptor: K-major operand, 128B swizzle, rows of 128
@@ -74,13 +91,13 @@ __device__ __forceinline__ uint64_t sw128_desc(const void *tile) {
 }
 
 // Instruction descriptor, kind::f16: fp32 accumulate, A and B of the same
-// 16-bit type, both K-major, M = 128, N = 256.
-__host__ __device__ constexpr uint32_t idesc_f16(bool bf16) {
+// 16-bit type, both K-major, M = 128 (256 for a pair), N = bn.
+__host__ __device__ constexpr uint32_t idesc_f16(bool bf16, int m, int bn) {
     return (1u << 4)                                    // D: f32
            | ((bf16 ? 1u : 0u) << 7)                    // A type
            | ((bf16 ? 1u : 0u) << 10)                   // B type
-           | (static_cast<uint32_t>(kBN >> 3) << 17)    // N / 8
-           | (static_cast<uint32_t>(kBM >> 4) << 24);   // M / 16
+           | (static_cast<uint32_t>(bn >> 3) << 17)     // N / 8
+           | (static_cast<uint32_t>(m >> 4) << 24);     // M / 16
 }
 
 __device__ __forceinline__ uint32_t ordered_bits_tc(float s) {
@@ -197,7 +214,7 @@ template <int LIST>
 __global__ void __launch_bounds__(kThreads, 1)
     retrieve_tc_kernel(const __grid_constant__ CUtensorMap tmap_q,
                        const __grid_constant__ CUtensorMap tmap_k, int64_t M, int dim,
-                       int n_queries, int q0, int nq, int a_rows, bool bf16,
+                       int n_queries, int q0, int nq, int a_rows, Ring ring, bool bf16,
                        unsigned long long *__restrict__ partial) {
     extern __shared__ __align__(1024) uint8_t smem_raw[];
     Smem &sm = *reinterpret_cast<Smem *>(
@@ -205,15 +222,17 @@ __global__ void __launch_bounds__(kThreads, 1)
     const int warp = threadIdx.x >> 5;
     const int lane = threadIdx.x & 31;
     const int nhalf = nq > kBM ? 2 : 1;
-    // accumulator columns: one query half x 256 keys = 256 columns, so a single half is
+    // accumulator columns: one query half x up to 256 keys = 256 columns, so a single half is
     // double-buffered (the argmax of a tile overlaps the next tile's MMAs) and two halves
     // fill all 512 columns with one buffer
     const int nbuf = nhalf == 1 ? 2 : 1;
     const int nkb = (dim + kBK - 1) / kBK;
-    const int64_t ntiles = (M + kBN - 1) / kBN;
+    const int bn = ring.bn;
+    const int64_t ntiles = (M + bn - 1) / bn;
+    const uint32_t b_off = nhalf * ring.a_bytes, stage_bytes = b_off + bn * kRowBytes;
 
     if (threadIdx.x == 0) {
-        for (int s = 0; s < kStages; ++s) {
+        for (int s = 0; s < ring.stages; ++s) {
             mbar_init(&sm.full[s], 1);
             mbar_init(&sm.empty[s], 1);
         }
@@ -236,34 +255,37 @@ __global__ void __launch_bounds__(kThreads, 1)
     if (warp == 0) {
         // ---------------- TMA producer ----------------
         if (lane == 0) {
-            uint32_t g = 0;
+            int s = 0;
+            uint32_t phase = 0;
+            int64_t issued = 0;
             bool alive = true;
             for (int64_t tile = blockIdx.x; tile < ntiles && alive; tile += gridDim.x) {
-                for (int kb = 0; kb < nkb; ++kb, ++g) {
-                    const int s = g % kStages;
-                    const uint32_t use = g / kStages;
-                    if (!wait_or_abort(&sm.empty[s], (use & 1u) ^ 1u, sm)) {
+                for (int kb = 0; kb < nkb; ++kb, ++issued) {
+                    if (!wait_or_abort(&sm.empty[s], phase ^ 1u, sm)) {
                         alive = false;
                         break;
                     }
-                    mbar_arrive_expect_tx(&sm.full[s], static_cast<uint32_t>(nhalf * a_rows * kBK * 2) + kBBytes);
+                    uint8_t *st = sm.ring + s * stage_bytes;
+                    mbar_arrive_expect_tx(&sm.full[s], (nhalf * a_rows + bn) * kRowBytes);
                     for (int h = 0; h < nhalf; ++h)
-                        tma_load_2d(sm.a[s][h], &tmap_q, kb * kBK, q0 + h * kBM, &sm.full[s]);
-                    tma_load_2d(sm.b[s], &tmap_k, kb * kBK, static_cast<int32_t>(tile * kBN),
-                                &sm.full[s]);
+                        tma_load_2d(st + h * ring.a_bytes, &tmap_q, kb * kBK, q0 + h * kBM, &sm.full[s]);
+                    tma_load_2d(st + b_off, &tmap_k, kb * kBK, static_cast<int32_t>(tile * bn), &sm.full[s]);
+                    if (++s == ring.stages) {
+                        s = 0;
+                        phase ^= 1u;
+                    }
                 }
             }
             // Drain: every issued stage must have landed before the CTA may exit.
-            const uint32_t issued = g;
-            for (uint32_t g2 = (issued > kStages ? issued - kStages : 0); g2 < issued; ++g2)
-                mbar_wait(&sm.full[g2 % kStages], (g2 / kStages) & 1u);
+            for (int64_t g = issued > ring.stages ? issued - ring.stages : 0; g < issued; ++g)
+                mbar_wait(&sm.full[g % ring.stages], static_cast<uint32_t>((g / ring.stages) & 1));
         }
     } else if (warp == 1) {
         // ---------------- MMA issuer ----------------
         if (lane == 0) {
-            const uint32_t idesc = idesc_f16(bf16);
-            uint32_t g = 0;
-            int it = 0;
+            const uint32_t idesc = idesc_f16(bf16, kBM, bn);
+            int s = 0, it = 0;
+            uint32_t phase = 0;
             bool alive = true;
             for (int64_t tile = blockIdx.x; tile < ntiles && alive; tile += gridDim.x, ++it) {
                 const int acc = it % nbuf;
@@ -271,22 +293,26 @@ __global__ void __launch_bounds__(kThreads, 1)
                 if (!wait_or_abort(&sm.acc_empty[acc], (ause & 1u) ^ 1u, sm)) break;
                 tc_fence_after();
                 const uint32_t d0 = tmem + static_cast<uint32_t>(acc * kBN);
-                for (int kb = 0; kb < nkb; ++kb, ++g) {
-                    const int s = g % kStages;
-                    if (!wait_or_abort(&sm.full[s], (g / kStages) & 1u, sm)) {
+                for (int kb = 0; kb < nkb; ++kb) {
+                    if (!wait_or_abort(&sm.full[s], phase, sm)) {
                         alive = false;
                         break;
                     }
                     tc_fence_after();
-                    const uint64_t bdesc = sw128_desc(sm.b[s]);
+                    const uint8_t *st = sm.ring + s * stage_bytes;
+                    const uint64_t bdesc = sw128_desc(st + b_off);
 #pragma unroll
                     for (int k = 0; k < kBK / 16; ++k) {
                         // advancing K by 16 elements = 32 bytes = 2 in the address field
                         for (int h = 0; h < nhalf; ++h)
-                            tc_mma_f16(d0 + h * kBN, sw128_desc(sm.a[s][h]) + 2 * k, bdesc + 2 * k,
-                                       idesc, kb > 0 || k > 0);
+                            tc_mma_f16(d0 + h * kBN, sw128_desc(st + h * ring.a_bytes) + 2 * k, bdesc + 2 * k, idesc,
+                                       kb > 0 || k > 0);
                     }
                     tc_commit(&sm.empty[s]);
+                    if (++s == ring.stages) {
+                        s = 0;
+                        phase ^= 1u;
+                    }
                 }
                 if (alive) tc_commit(&sm.acc_full[acc]);
             }
@@ -311,9 +337,10 @@ __global__ void __launch_bounds__(kThreads, 1)
                 ok = __shfl_sync(0xffffffffu, ok, 0);
                 if (!ok) break;
                 tc_fence_after();
-                const int64_t row0 = tile * kBN;
+                const int64_t row0 = tile * bn;
+                // a quarter without queries only hands its buffer back
 #pragma unroll 1
-                for (int c0 = 0; c0 < kBN; c0 += 32) {
+                for (int c0 = 0; c0 < bn && h * kBM + quarter * 32 < nq; c0 += 32) {
                     float v[32];
                     tmem_ld32(tmem + (static_cast<uint32_t>(quarter * 32) << 16) +
                                   static_cast<uint32_t>(acc * kBN + h * kBN + c0),
@@ -358,8 +385,7 @@ __global__ void __launch_bounds__(kThreads, 1)
 // and 2p + 1 (no row) for their queries, so the finalize reads as many slots as after
 // the single-CTA kernel on the same grid.
 constexpr int kPairThreads = 6 * 32;
-constexpr uint32_t kPairRows = kBN / 2;                              // key rows per CTA and tile
-constexpr uint32_t kPairStageBytes = kABytes + kPairRows * kBK * 2;  // per CTA: 16 KB + 16 KB
+constexpr uint32_t kPairRows = kBN / 2;   // key rows per CTA and tile, at most
 
 template <int LIST>
 struct PairSmem {
@@ -376,17 +402,11 @@ struct PairSmem {
     float epi[kScratchRows][33];
 };
 
-// kind::f16 instruction descriptor of the pair MMA: M = 256 (128 rows per CTA), N = 256.
-__host__ __device__ constexpr uint32_t idesc_f16_pair(bool bf16) {
-    return (1u << 4) | ((bf16 ? 1u : 0u) << 7) | ((bf16 ? 1u : 0u) << 10) |
-           (static_cast<uint32_t>(kBN >> 3) << 17) | (static_cast<uint32_t>((2 * kBM) >> 4) << 24);
-}
-
 template <int LIST>
 __global__ void __launch_bounds__(kPairThreads, 1)
     retrieve_tc_pair_kernel(const __grid_constant__ CUtensorMap tmap_q,
                             const __grid_constant__ CUtensorMap tmap_k, int64_t M, int dim, int n_queries,
-                            int q0, int nq, bool bf16, unsigned long long *__restrict__ partial) {
+                            int q0, int nq, int bn, bool bf16, unsigned long long *__restrict__ partial) {
     using Sm = PairSmem<LIST>;
     constexpr int S = Sm::kStages;
     extern __shared__ __align__(1024) uint8_t smem_raw[];
@@ -397,7 +417,7 @@ __global__ void __launch_bounds__(kPairThreads, 1)
     const int64_t pair = blockIdx.x >> 1;
     const int64_t npairs = gridDim.x >> 1;
     const int nkb = (dim + kBK - 1) / kBK;
-    const int64_t ntiles = (M + kBN - 1) / kBN;
+    const int64_t ntiles = (M + bn - 1) / bn;
 
     if (threadIdx.x == 0) {
         for (int s = 0; s < S; ++s) {
@@ -434,11 +454,11 @@ __global__ void __launch_bounds__(kPairThreads, 1)
                         alive = false;
                         break;
                     }
-                    if (rank == 0) mbar_arrive_expect_tx(&sm.full[s], 2 * kPairStageBytes);
+                    if (rank == 0) mbar_arrive_expect_tx(&sm.full[s], 2 * kABytes + bn * kRowBytes);
                     const uint32_t full0 = mapa_shared(&sm.full[s], 0);
                     tma_load_2d_pair(sm.a[s], &tmap_q, kb * kBK, q0 + static_cast<int>(rank) * kBM, full0);
                     tma_load_2d_pair(sm.b[s], &tmap_k, kb * kBK,
-                                     static_cast<int32_t>(tile * kBN + rank * kPairRows), full0);
+                                     static_cast<int32_t>(tile * bn + rank * (bn / 2)), full0);
                 }
             }
             // Before the CTA may exit: every issued stage landed (the even CTA's full
@@ -454,7 +474,7 @@ __global__ void __launch_bounds__(kPairThreads, 1)
     } else if (warp == 1) {
         // ---------------- MMA issuer (even CTA) ----------------
         if (rank == 0 && lane == 0) {
-            const uint32_t idesc = idesc_f16_pair(bf16);
+            const uint32_t idesc = idesc_f16(bf16, 2 * kBM, bn);
             uint32_t g = 0;
             int it = 0;
             bool alive = true;
@@ -499,10 +519,10 @@ __global__ void __launch_bounds__(kPairThreads, 1)
             ok = __shfl_sync(0xffffffffu, ok, 0);
             if (!ok) break;
             tc_fence_after();
-            // column c of the accumulator is key row tile * 256 + c (the even CTA's 128 rows first)
-            const int64_t row0 = tile * kBN;
+            // column c of the accumulator is key row tile * bn + c (the even CTA's half first)
+            const int64_t row0 = tile * bn;
 #pragma unroll 1
-            for (int c0 = 0; c0 < kBN; c0 += 32) {
+            for (int c0 = 0; c0 < bn; c0 += 32) {
                 float v[32];
                 tmem_ld32(tmem + (static_cast<uint32_t>(quarter * 32) << 16) + static_cast<uint32_t>(acc * kBN + c0),
                           v);
@@ -527,6 +547,21 @@ __global__ void __launch_bounds__(kPairThreads, 1)
         tc_fence_after();
         tmem_dealloc_pair(tmem, kTmemCols);
     }
+}
+
+// Key rows per tile for `ctas` CTAs (or pairs) that take tiles in turn: the fewest rounds of
+// full tiles, and the height that spreads the rows evenly over them (in steps of 32, one TMEM
+// load of the epilogue). With 256 rows throughout, 80,000 rows were 2.06 tiles per CTA and took
+// three rounds, and an index of a few thousand rows ran on a few CTAs. Top-1 of one query with
+// its merge, us, 256 rows -> now: 2,000 x 384 11.5 -> 9.1, 10,000 x 384 12.0 -> 10.3, 45,000 x 768
+// 19.4 -> 17.4, 80,000 x 768 30.5 -> 25.8, 200,000 x 768 54.3 -> 49.6, 1,000,000 x 768 215 -> 215;
+// of 256 queries on SM pairs: 2,000 x 384 15.9 -> 11.1, 100,000 x 768 41.0 -> 39.4. Heights
+// below 64 were slower again (2,000 x 768 in 32 rows 11.5 us, in 64 9.9 to 12.2; 10,000 x 1024
+// 18.9, 14.6): every CTA fetches the queries.
+int tile_rows(int64_t M, int ctas) {
+    const int64_t rounds = (M + static_cast<int64_t>(kBN) * ctas - 1) / (static_cast<int64_t>(kBN) * ctas);
+    const int64_t rows = (M + rounds * ctas - 1) / (rounds * ctas);
+    return static_cast<int>(rows <= kMinRows ? kMinRows : (rows + 31) / 32 * 32);
 }
 
 bool make_map(CUtensorMap *map, const void *base, int64_t rows, int dim, bool bf16, int box_rows) {
@@ -565,10 +600,10 @@ static_assert(sizeof(Smem) + 1024 <= 227 * 1024, "the ring and scratch must fit 
 static_assert(sizeof(PairSmem<1>) + 1024 <= 227 * 1024, "the pair ring must fit one CTA's shared memory");
 static_assert(sizeof(PairSmem<8>) + 1024 <= 227 * 1024, "the pair ring and scratch must fit one CTA's shared memory");
 
-size_t retrieve_tc_smem_bytes() { return sizeof(Smem) + 1024; }
-
+// CTAs of a launch: one per SM, or per tile of kMinRows rows; never more parts than a GEMV's over
+// the same rows (the workspace's size).
 int retrieve_tc_grid(int64_t M, int sms) {
-    const int64_t ntiles = (M + kBN - 1) / kBN;
+    const int64_t ntiles = (M + kMinRows - 1) / kMinRows;
     return static_cast<int>(ntiles < 1 ? 1 : (ntiles < sms ? ntiles : sms));
 }
 
@@ -581,18 +616,19 @@ cudaError_t launch_tc(const RetrieveParams &p, int grid, cudaStream_t stream, ui
     // swizzle atom); the rest of the A tile is never read back (its TMEM lanes belong to
     // no query), and copies that are mostly out of bounds are slow.
     const int a_rows = p.n_queries >= kBM ? kBM : ((p.n_queries + 7) & ~7);
-    if (!make_map(&tq, p.queries, p.n_queries, p.dim, bf16, a_rows) ||
-        !make_map(&tk, p.index, p.M > 0 ? p.M : 1, p.dim, bf16, kBN))
+    const int bn = tile_rows(p.M, grid);
+    if (!make_map(&tq, p.queries, p.n_queries, p.dim, bf16, a_rows) || !make_map(&tk, p.index, p.M, p.dim, bf16, bn))
         return cudaErrorInvalidValue;
-    const int smem = static_cast<int>(retrieve_tc_smem_bytes());
+    const int smem = static_cast<int>(sizeof(Smem) + 1024);
     cudaError_t e = ensure_smem(reinterpret_cast<const void *>(retrieve_tc_kernel<LIST>), smem);
     if (e != cudaSuccess) return e;
     // Passes of more than 128 queries run on SM pairs when the grid splits into pairs.
     const bool pairs = grid % 2 == 0 && p.n_queries > kBM;
     CUtensorMap tk_pair;
+    const int bn_pair = pairs ? tile_rows(p.M, grid / 2) : 0;
     const int smem_pair = static_cast<int>(sizeof(PairSmem<LIST>) + 1024);
     if (pairs) {
-        if (!make_map(&tk_pair, p.index, p.M, p.dim, bf16, static_cast<int>(kPairRows))) return cudaErrorInvalidValue;
+        if (!make_map(&tk_pair, p.index, p.M, p.dim, bf16, bn_pair / 2)) return cudaErrorInvalidValue;
         e = ensure_smem(reinterpret_cast<const void *>(retrieve_tc_pair_kernel<LIST>), smem_pair);
         if (e != cudaSuccess) return e;
     }
@@ -613,10 +649,17 @@ cudaError_t launch_tc(const RetrieveParams &p, int grid, cudaStream_t stream, ui
             cfg.attrs = attr;
             cfg.numAttrs = 1;
             e = cudaLaunchKernelEx(&cfg, retrieve_tc_pair_kernel<LIST>, tq, tk_pair, p.M, p.dim, p.n_queries, q0,
-                                   nq, bf16, partial);
+                                   nq, bn_pair, bf16, partial);
         } else {
+            Ring ring;
+            ring.bn = bn;
+            // the A tile of a launch with few queries (its tensor map's box) needs no more rows
+            ring.a_bytes = a_rows <= kFewQueries ? kFewQueries * kRowBytes : kABytes;
+            const int fit = static_cast<int>(kRingBytes / ((nq > kBM ? 2 : 1) * ring.a_bytes + bn * kRowBytes));
+            const int deep = static_cast<int>(kKeyBytes / (bn * kRowBytes));
+            ring.stages = fit < deep ? fit : deep;
             retrieve_tc_kernel<LIST><<<grid, kThreads, smem, stream>>>(tq, tk, p.M, p.dim, p.n_queries, q0, nq,
-                                                                       a_rows, bf16, partial);
+                                                                       a_rows, ring, bf16, partial);
             e = cudaGetLastError();
         }
         if (e != cudaSuccess) return e;

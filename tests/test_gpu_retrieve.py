@@ -178,3 +178,36 @@ def test_tensor_core_ties_and_nan_rows(cuda_device):
     for q in range(Q):
         assert idx[q] == min(r for qq, r in planted if qq == q)
     assert np.all(np.isfinite(score))
+
+
+@pytest.mark.parametrize("dtype_name", ["float16", "bfloat16"])
+@pytest.mark.parametrize("M,dim", [(1, 8), (63, 64), (65, 200), (130, 4096), (9729, 64), (38912, 72), (38913, 64),
+                                   (50000, 64)])
+@pytest.mark.parametrize("Q", [1, 32, 33, 129, 257])
+def test_tile_heights(cuda_device, dtype_name, M, dim, Q):
+    """Tiles of 16-bit keys are as tall as spreads the rows evenly over the rounds: one tile of
+    64 rows, heights between the limits (of SM pairs too), CTAs without a tile, the last row
+    of a round, A tiles of 32 and 128 rows and rings of every depth, several rounds of the
+    ring and of the two accumulators. Small integers: exact scores and many ties."""
+    import torch
+    import paper_2608_02560_gb300 as pg
+    rng = np.random.default_rng(M + dim + Q)
+    index = rng.integers(-2, 3, size=(M, dim)).astype(np.float32)
+    queries = rng.integers(-2, 3, size=(Q, dim)).astype(np.float32)
+    dtype = getattr(torch, dtype_name)
+    ix, qs = (torch.from_numpy(a).to(cuda_device, dtype) for a in (index, queries))
+    scores = queries @ index.T                 # exact: |sum| <= 4 * 4096
+    order = np.argsort(-scores, axis=1, kind="stable")
+    i1 = torch.empty(Q, dtype=torch.int64, device=cuda_device)
+    s1 = torch.empty(Q, dtype=torch.float32, device=cuda_device)
+    pg.precog_retrieve(ix, qs, i1, s1)
+    np.testing.assert_array_equal(i1.cpu().numpy(), order[:, 0])
+    for k in (2, 5):
+        i = torch.empty((Q, k), dtype=torch.int64, device=cuda_device)
+        s = torch.empty((Q, k), dtype=torch.float32, device=cuda_device)
+        pg.precog_retrieve_topk(ix, qs, k, i, s)
+        m = min(k, M)
+        np.testing.assert_array_equal(i.cpu().numpy()[:, :m], order[:, :m])
+        np.testing.assert_array_equal(s.cpu().numpy()[:, :m], np.take_along_axis(scores, order[:, :m], axis=1))
+        assert (i[:, m:] == -1).all()
+    assert pg.precog_device_status()[0] == 0
