@@ -346,14 +346,95 @@ constexpr int kFormPower = 2;     // and A_re[n] = (n+1) A_re[0]: alpha_n = m (m
 template <bool HAS_Y>
 constexpr int block_channels() { return HAS_Y ? 128 : 256; }
 
-template <typename TIn, bool HAS_Y, bool HAS_H0>
+// ---- chunks split over the CTAs of a cluster (captures with few work items) ----
+// As in the real scan: a chunk's final state is the sum over its segments of the segment's
+// own final state (from zero) decayed by the tokens after it, h = sum_s exp(A * dt_s) h_s with
+// dt_s the dt summed over the segments after s. The decay's phase A_im * dt_s may be many
+// turns, so dt is summed to twice fp32 precision and the phase formed as a two-float product.
+struct DtSum {
+    float hi, lo;
+    __device__ __forceinline__ void add(float v) {   // Knuth's two-sum
+        const float s = hi + v, b = s - hi;
+        lo += (hi - (s - b)) + (v - b);
+        hi = s;
+    }
+};
+
+template <int CB>
+struct SplitState {
+    int32_t dead;               // this CTA gave up on a wait
+    alignas(16) float4 h[kN / 2][CB];   // states 2i, 2i+1 of a channel as (re, im, re, im)
+    float2 dt[CB];
+};
+
+template <int CB>
+__device__ __forceinline__ void combine(unsigned char *buf, const ScanParams &p, bool dead, bool live, int W,
+                                        const float (&hr)[kN], const float (&hi)[kN], DtSum dt, int64_t chunk,
+                                        int layer, int d0) {
+    SplitState<CB> &sm = *reinterpret_cast<SplitState<CB> *>(buf);
+    const int tid = threadIdx.x, segs = p.segments;
+    if (tid == 0) sm.dead = dead;
+    if (live) {
+        sm.dt[tid] = make_float2(dt.hi, dt.lo);
+#pragma unroll
+        for (int i = 0; i < kN / 2; ++i)
+            sm.h[i][tid] = make_float4(hr[2 * i], hi[2 * i], hr[2 * i + 1], hi[2 * i + 1]);
+    }
+    cluster_sync_all();
+    bool any_dead = false;
+    for (int s = 0; s < segs; ++s) any_dead |= ld_cluster_u32(mapa_shared(&sm.dead, s)) != 0u;
+    for (int i = static_cast<int>(cluster_ctarank()) * CB + tid; i < kN / 2 * W && !any_dead; i += segs * CB) {
+        const int q = i / W, ch = i % W;
+        const int64_t row = static_cast<int64_t>(layer) * p.D + d0 + ch;
+        const float4 a = reinterpret_cast<const float4 *>(p.A)[row * (kN / 2) + q];
+        const f2 ar = pack2(a.x * kLog2e, a.z * kLog2e), ai = pack2(a.y, a.w);
+        DtSum after{0.f, 0.f};
+        f2 sr = 0, si = 0;
+        for (int s = segs - 1; s >= 0; --s) {
+            const float4 v = ld_cluster_f4(mapa_shared(&sm.h[q][ch], s));
+            const f2 vr = pack2(v.x, v.z), vi = pack2(v.y, v.w), dd = pack2(after.hi, after.hi);
+            float e0, e1;
+            unpack2(mul2(dd, ar), e0, e1);
+            const f2 mag = pack2(ex2(e0), ex2(e1));
+            const f2 th = mul2(dd, ai);
+            float t0, t1;
+            unpack2(th, t0, t1);
+            const f2 tl = fma2(pack2(after.lo, after.lo), ai, fma2(dd, ai, pack2(-t0, -t1)));
+            f2 sn, cs;
+            sincos_pair(th, tl, sn, cs);
+            const f2 fr = mul2(mag, cs), fi = mul2(mag, sn);
+            float i0, i1;
+            unpack2(vi, i0, i1);
+            sr = fma2(fr, vr, fma2(fi, pack2(-i0, -i1), sr));
+            si = fma2(fr, vi, fma2(fi, vr, si));
+            const uint32_t at = mapa_shared(&sm.dt[ch], s);
+            after.add(__uint_as_float(ld_cluster_u32(at)));
+            after.lo += __uint_as_float(ld_cluster_u32(at + 4));
+        }
+        float r0, r1, i0, i1;
+        unpack2(sr, r0, r1);
+        unpack2(si, i0, i1);
+        const int64_t off = ((chunk * p.L_out + p.layer0 + layer) * static_cast<int64_t>(p.D) + d0 + ch) * kN + 2 * q;
+        if (p.state_dtype == PRECOG_F32) {
+            *reinterpret_cast<float4 *>(static_cast<float *>(p.states) + 2 * off) = make_float4(r0, i0, r1, i1);
+        } else {
+            const __nv_bfloat162 lo = __floats2bfloat162_rn(r0, i0), up = __floats2bfloat162_rn(r1, i1);
+            *reinterpret_cast<uint2 *>(static_cast<__nv_bfloat16 *>(p.states) + 2 * off) =
+                make_uint2(*reinterpret_cast<const uint32_t *>(&lo), *reinterpret_cast<const uint32_t *>(&up));
+        }
+    }
+    cluster_sync_all();   // no CTA leaves while another may still read its shared memory
+}
+
+template <typename TIn, bool HAS_Y, bool HAS_H0, bool SPLIT>
 __global__ void __launch_bounds__(block_channels<HAS_Y>())
     scan_complex_kernel(const ScanParams p, const int cblocks) {
     constexpr int CB = block_channels<HAS_Y>();
     constexpr int SZ = static_cast<int>(sizeof(TIn));
     extern __shared__ __align__(128) unsigned char smem_raw[];
     CSmem<TIn, CB> &sm = *reinterpret_cast<CSmem<TIn, CB> *>(smem_raw);
-    int64_t item = blockIdx.x;
+    static_assert(!SPLIT || (!HAS_Y && !HAS_H0 && sizeof(SplitState<CB>) <= sizeof(sm.tile)), "the states fit the ring");
+    int64_t item = SPLIT ? blockIdx.x / p.segments : blockIdx.x;
     const int cb = static_cast<int>(item % cblocks);
     item /= cblocks;
     const int64_t chunk = p.order ? p.order[item % p.n_chunks] : item % p.n_chunks;
@@ -380,6 +461,14 @@ __global__ void __launch_bounds__(block_channels<HAS_Y>())
             return;
         }
         len = end - start;
+    }
+    DtSum dt_sum{0.f, 0.f};
+    if constexpr (SPLIT) {
+        // this CTA's share of the chunk: whole tiles (the cluster's CTAs left together above)
+        const int64_t share = ((len + kCT - 1) / kCT + p.segments - 1) / p.segments * kCT;
+        const int64_t skip = share * cluster_ctarank();
+        start += skip;
+        len = len > skip ? (len - skip < share ? len - skip : share) : 0;
     }
     const TIn *xl = static_cast<const TIn *>(p.x) + layer * p.ls_xd;
     const TIn *dtl = static_cast<const TIn *>(p.dt) + layer * p.ls_xd;
@@ -519,6 +608,7 @@ __global__ void __launch_bounds__(block_channels<HAS_Y>())
         return true;
     };
 
+    bool dead = false;   // a wait ran out (split: the cluster's other CTAs still expect this one)
     if (!HAS_Y && form == kFormPower) {
         // rescaled capture: running exponent and phase, tokens since the last
         // renormalisation (the same count on every lane), the live lanes of this warp
@@ -529,6 +619,7 @@ __global__ void __launch_bounds__(block_channels<HAS_Y>())
             const float xv = to_f32(tl.x[t * W + tid]);
             const float dv = to_f32(tl.dt[t * W + tid]);
             const float u = dv * xv;
+            if constexpr (SPLIT) dt_sum.add(dv);
             float b[kN];
             widen_row<float>(b_row(tl, t), b);
             const f2 uu = pack2(u, u);
@@ -555,7 +646,8 @@ __global__ void __launch_bounds__(block_channels<HAS_Y>())
             phc = ph;
             ++since;
         });
-        if (!done) return;
+        if (!done && !SPLIT) return;
+        dead = !done;
         if (live) renormalise_c(hr, hi, Lc, phc);
     } else if (!HAS_Y && form == kFormHarmonic) {
         // rescaled capture, harmonic form: running sum of dt and phase; the window on the
@@ -574,6 +666,7 @@ __global__ void __launch_bounds__(block_channels<HAS_Y>())
             const float xv = to_f32(tl.x[t * W + tid]);
             const float dv = to_f32(tl.dt[t * W + tid]);
             const float u = dv * xv;
+            if constexpr (SPLIT) dt_sum.add(dv);
             float b[kN];
             widen_row<float>(b_row(tl, t), b);
             const float th = dv * a1, tle = fmaf(dv, a1, -th);
@@ -599,13 +692,15 @@ __global__ void __launch_bounds__(block_channels<HAS_Y>())
             phc = ph;
             ++since;
         });
-        if (!done) return;
+        if (!done && !SPLIT) return;
+        dead = !done;
         if (live) renormalise_h(hr, hi, ar, Sc, phc);
     } else {
         const bool done = scan_tiles([&](const CTile<TIn, CB> &tl, int t, int64_t k) {
             const float xv = to_f32(tl.x[t * W + tid]);
             const float dv = to_f32(tl.dt[t * W + tid]);
             const float u = dv * xv;
+            if constexpr (SPLIT) dt_sum.add(dv);
             float b[kN], cr[kN];
             widen_row<float>(b_row(tl, t), b);
             if constexpr (HAS_Y) widen_row<float>(c_row(tl, t), cr);
@@ -650,7 +745,13 @@ __global__ void __launch_bounds__(block_channels<HAS_Y>())
                 else static_cast<__nv_bfloat16 *>(p.y)[yo] = __float2bfloat16_rn(y);
             }
         });
-        if (!done) return;
+        if (!done && !SPLIT) return;
+        dead = !done;
+    }
+    if constexpr (SPLIT) {
+        __syncthreads();
+        combine<CB>(reinterpret_cast<unsigned char *>(sm.tile), p, dead, live, W, hr, hi, dt_sum, chunk, layer, d0);
+        return;
     }
     if (p.states && live) {
         const int64_t off = ((chunk * p.L_out + p.layer0 + layer) * static_cast<int64_t>(D) + d) * kN;
@@ -664,6 +765,19 @@ __global__ void __launch_bounds__(block_channels<HAS_Y>())
     }
 }
 
+// CTAs per chunk of a capture (1: not split): 8 or 4, within one wave of two CTAs per SM. An
+// unsplit launch takes 0.24 us (power form) to 0.4 us (per-index) per token of its chunks while
+// the SMs hold it: 1 x 1 x 4000 tokens 946 -> 140 us, 1 x 8 x 3000 712 -> 108, 24 layers x 3 x 500
+// 128 -> 68, 24 x 1 x 200 57 -> 27 (per-index fp32 1580 -> 223, 1188 -> 170, 207 -> 123, 88 -> 37).
+// Two shares gain little (24 x 6 x 500: 128 -> 121) or lose (fp32 209 -> 233), and so do short
+// chunks (2 x 10 x 100 x 1000 channels: 39 -> 43, fp32 54 -> 76).
+int split_segments(const ScanParams &p, int64_t items) {
+    const int64_t slots = 2 * static_cast<int64_t>(device_sm_count());
+    const int64_t tokens = p.T_tot / p.n_chunks;   // on average
+    if (items * 8 <= slots && tokens >= 8 * kCT) return 8;
+    return items * 4 <= slots && tokens >= 4 * kCT ? 4 : 1;
+}
+
 template <typename TIn, bool HAS_Y, bool HAS_H0>
 cudaError_t launch_c(const ScanParams &p, cudaStream_t stream) {
     constexpr int CB = block_channels<HAS_Y>();
@@ -672,8 +786,34 @@ cudaError_t launch_c(const ScanParams &p, cudaStream_t stream) {
     if (items == 0) return cudaSuccess;
     if (items > 0x7fffffffLL) return cudaErrorInvalidConfiguration;
     const int smem = static_cast<int>(sizeof(CSmem<TIn, CB>));
-    auto kern = scan_complex_kernel<TIn, HAS_Y, HAS_H0>;
-    cudaError_t e = ensure_smem(reinterpret_cast<const void *>(kern), smem);
+    cudaError_t e;
+    if constexpr (!HAS_Y && !HAS_H0) {
+        const int segs = split_segments(p, items);
+        if (segs > 1) {
+            auto kern = scan_complex_kernel<TIn, false, false, true>;
+            e = ensure_smem(reinterpret_cast<const void *>(kern), smem);
+            if (e != cudaSuccess) return e;
+            ScanParams q = p;
+            q.segments = segs;
+            cudaLaunchConfig_t cfg = {};
+            cfg.gridDim = dim3(static_cast<unsigned>(items * segs));   // at most two per SM
+            cfg.blockDim = dim3(CB);
+            cfg.dynamicSmemBytes = static_cast<size_t>(smem);
+            cfg.stream = stream;
+            cudaLaunchAttribute attr[1];
+            attr[0].id = cudaLaunchAttributeClusterDimension;
+            attr[0].val.clusterDim.x = static_cast<unsigned>(segs);
+            attr[0].val.clusterDim.y = 1;
+            attr[0].val.clusterDim.z = 1;
+            cfg.attrs = attr;
+            cfg.numAttrs = 1;
+            e = cudaLaunchKernelEx(&cfg, kern, q, cblocks);
+            if (e == cudaSuccess) count_launches(1);
+            return e;
+        }
+    }
+    auto kern = scan_complex_kernel<TIn, HAS_Y, HAS_H0, false>;
+    e = ensure_smem(reinterpret_cast<const void *>(kern), smem);
     if (e != cudaSuccess) return e;
     kern<<<static_cast<unsigned>(items), CB, smem, stream>>>(p, cblocks);
     e = cudaGetLastError();

@@ -289,3 +289,46 @@ def test_complex_rescaled_capture_regimes(cuda_device, form, regime):
         sl = slice(q * Tq, (q + 1) * Tq)
         ref, _ = oracle.scan_complex(xq[sl], dtq[sl], A.real, A.imag, Bq[sl], [0, Tq], h0=h0)
         assert _cplx_err(h[q, 0].cpu().numpy(), ref[0]) < TOL_BF16
+
+
+@pytest.mark.parametrize("in16", [False, True])
+@pytest.mark.parametrize("form", FORMS)
+@pytest.mark.parametrize("D,lens", [(64, [2500]), (256, [130]), (600, [0, 900, 33, 128, 129]), (8, [85, 700]),
+                                    (256, [137] * 70)])
+def test_complex_split_chunks(cuda_device, D, lens, form, in16):
+    """Captures with few work items share each chunk's tokens among a cluster's CTAs and
+    combine their states: 2, 4 and 8 shares, shares without tokens, chunks shorter than the
+    shares, bf16 states. Slow decays (small dt in the second half) keep the early segments'
+    states and their many turns of phase in the result, and with them the per-token rounding
+    of every form (1e-5 and more over 2500 tokens), so the bound is the unsplit scan's own
+    error (the state-only prefill from the zero state), which the combination adds one
+    rounding per segment to, or the usual tolerance where that is larger."""
+    import torch
+    pg = _pg()
+    in_dtype = torch.bfloat16 if in16 else None
+    offsets = np.concatenate([[0], np.cumsum(lens)]).astype(np.int64)
+    T = int(offsets[-1])
+    x, dt, _, B, C = synth.host_scan_inputs(T, D, 16, seed=D + T)
+    dt[T // 2:] *= 0.02
+    if in16:
+        rnd = lambda a: torch.from_numpy(a).to(torch.bfloat16).float().numpy()
+        x, dt, B = rnd(x), rnd(dt), rnd(B)
+    A = _complex_A(D, 16, D, form)
+    tol = TOL_BF16 if in16 else TOL_F32
+    hs, _ = _encode(pg, cuda_device, x, dt, B, C, A, offsets, with_y=False, in_dtype=in_dtype)
+    ref_h, _ = oracle.scan_complex(x, dt, A.real, A.imag, B, offsets)
+    pg_in = lambda a: _t(a, cuda_device, in_dtype)
+    bank = torch.zeros((1, 1, D, 16), dtype=torch.complex64, device=cuda_device)
+    for c in range(len(lens)):
+        if lens[c] == 0:
+            assert np.all(hs[c] == 0)
+            continue
+        sl = slice(offsets[c], offsets[c + 1])
+        one = torch.empty((1, 1, D, 16), dtype=torch.complex64, device=cuda_device)
+        pg.precog_prefill_from_state(
+            pg.scan_inputs(pg_in(x[sl]), pg_in(dt[sl]), pg_in(B[sl]), _t(A, cuda_device), a_kind=pg.PRECOG_A_COMPLEX),
+            1, lens[c], bank, torch.tensor([-1], device=cuda_device), state_out=one)
+        unsplit = _cplx_err(one[0, 0].cpu().numpy(), ref_h[c])
+        assert _cplx_err(hs[c], ref_h[c]) < max(tol, 1.25 * unsplit)
+    half, _ = _encode(pg, cuda_device, x, dt, B, C, A, offsets, with_y=False, in_dtype=in_dtype, state_dtype="bf16")
+    assert rel_err_stored(half.real, hs.real) < 1e-7 and rel_err_stored(half.imag, hs.imag) < 1e-7
