@@ -153,6 +153,15 @@ __device__ __forceinline__ void tc_commit(uint64_t *bar) {
                      smem_u32(bar))
                  : "memory");
 }
+// ---- dependent launches ----
+// Wait until the stream's previous kernel has completed and its writes are visible: the first
+// statement of every thread of a kernel launched with launch_dependent, before any access to
+// global memory.
+__device__ __forceinline__ void grid_dependency_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+// Let the stream's next kernel, if it was launched dependent, become resident from here on.
+__device__ __forceinline__ void grid_dependency_launch() {
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
 // ---- CTA pairs (clusters of two CTAs sharing one tcgen05 MMA, cta_group::2) ----
 // A kernel uses one cta_group throughout: these are the pair forms of the
 // allocation, MMA and commit above.

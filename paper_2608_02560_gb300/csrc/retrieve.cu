@@ -171,6 +171,8 @@ __global__ void finalize_kernel(const unsigned long long *__restrict__ partial, 
                                 int n_queries, int64_t *__restrict__ best_idx,
                                 float *__restrict__ best_score, int64_t row_offset,
                                 int64_t *__restrict__ keys_out) {
+    grid_dependency_wait();
+    grid_dependency_launch();   // a prefill from the retrieved rows
     const int q = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const int lane = threadIdx.x & 31;
     if (q >= n_queries) return;
@@ -311,6 +313,8 @@ __device__ __forceinline__ unsigned long long warp_max_u64(unsigned long long v)
 __global__ void finalize_topk_kernel(const unsigned long long *__restrict__ partial, int n_parts, int log_used,
                                      int n_queries, int k, int64_t *__restrict__ best_idx,
                                      float *__restrict__ best_score) {
+    grid_dependency_wait();
+    grid_dependency_launch();   // a prefill from the retrieved rows
     constexpr int kAhead = 8;
     const int q = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const int lane = threadIdx.x & 31;
@@ -752,10 +756,9 @@ cudaError_t launch_retrieve(const RetrieveParams &p, cudaStream_t stream) {
         e = launch_gemv<float>(p, stream, parts, &launches);
     }
     if (e == cudaSuccess) {
-        finalize_kernel<<<(p.n_queries + 3) / 4, 128, 0, stream>>>(
-            static_cast<const unsigned long long *>(p.workspace), parts, p.n_queries, p.best_idx,
-            p.best_score, p.row_offset, p.keys_out);
-        e = cudaGetLastError();
+        e = launch_dependent(finalize_kernel, dim3((p.n_queries + 3) / 4), dim3(128), 0, stream,
+                             static_cast<const unsigned long long *>(p.workspace), parts, p.n_queries, p.best_idx,
+                             p.best_score, p.row_offset, p.keys_out);
         if (e == cudaSuccess) ++launches;
     }
     count_launches(launches);
@@ -799,10 +802,9 @@ cudaError_t launch_retrieve_topk(const RetrieveParams &p, int k, cudaStream_t st
         e = launch_gemv_topk<float>(p, stream, parts, &launches);
     }
     if (e == cudaSuccess) {
-        finalize_topk_kernel<<<(p.n_queries + 3) / 4, 128, 0, stream>>>(
-            static_cast<const unsigned long long *>(p.workspace), parts, log_used, p.n_queries, k, p.best_idx,
-            p.best_score);
-        e = cudaGetLastError();
+        e = launch_dependent(finalize_topk_kernel, dim3((p.n_queries + 3) / 4), dim3(128), 0, stream,
+                             static_cast<const unsigned long long *>(p.workspace), parts, log_used, p.n_queries, k,
+                             p.best_idx, p.best_score);
         if (e == cudaSuccess) ++launches;
     }
     count_launches(launches);

@@ -216,6 +216,7 @@ __global__ void __launch_bounds__(kThreads, 1)
                        const __grid_constant__ CUtensorMap tmap_k, int64_t M, int dim,
                        int n_queries, int q0, int nq, int a_rows, Ring ring, bool bf16,
                        unsigned long long *__restrict__ partial) {
+    grid_dependency_launch();   // the merge of the partial keys
     extern __shared__ __align__(1024) uint8_t smem_raw[];
     Smem &sm = *reinterpret_cast<Smem *>(
         (reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~static_cast<uintptr_t>(1023));
@@ -409,6 +410,7 @@ __global__ void __launch_bounds__(kPairThreads, 1)
                             int q0, int nq, int bn, bool bf16, unsigned long long *__restrict__ partial) {
     using Sm = PairSmem<LIST>;
     constexpr int S = Sm::kStages;
+    grid_dependency_launch();   // the merge of the partial keys
     extern __shared__ __align__(1024) uint8_t smem_raw[];
     Sm &sm = *reinterpret_cast<Sm *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~static_cast<uintptr_t>(1023));
     const int warp = threadIdx.x >> 5;

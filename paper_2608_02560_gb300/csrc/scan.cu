@@ -867,6 +867,7 @@ __device__ __forceinline__ void combine(unsigned char *buf, const ScanParams &p,
 template <class C>
 __global__ void __launch_bounds__(C::LB_THREADS, C::LB_BLOCKS)
     scan_kernel(const ScanParams p, const int DS_arg, const int slices, const __grid_constant__ SliceMaps maps) {
+    if constexpr (C::HAS_H0) grid_dependency_wait();
     using TIn = typename C::TIn;
     const int DS = C::FIXDS ? C::FIXDS : DS_arg;
     constexpr int CPT = C::CPT, TILE = C::TILE, STAGES = C::STAGES, SZ = C::SZ;
@@ -1314,6 +1315,9 @@ cudaError_t launch_cfg(const ScanParams &p, cudaStream_t stream) {
         cfg.attrs = attr;
         cfg.numAttrs = 1;
         e = cudaLaunchKernelEx(&cfg, kern, p, DS, slices, maps);
+    } else if constexpr (C::HAS_H0) {
+        // a prefill, usually behind the retrieval of its rows
+        e = launch_dependent(kern, dim3(static_cast<unsigned>(items)), dim3(DS / C::CPT), smem, stream, p, DS, slices, maps);
     } else {
         kern<<<static_cast<unsigned>(items), DS / C::CPT, smem, stream>>>(p, DS, slices, maps);
         e = cudaGetLastError();

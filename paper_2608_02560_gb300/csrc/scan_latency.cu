@@ -91,6 +91,7 @@ __device__ __forceinline__ void store_state4(void *base, int dtype, int64_t off,
 template <typename TIn, bool HAS_H0>
 __global__ void __launch_bounds__(kLThreads)
     scan_latency_kernel(const ScanParams p, const int cblocks) {
+    if constexpr (HAS_H0) grid_dependency_wait();
     extern __shared__ __align__(128) unsigned char smem_raw[];
     LatSmem<TIn> &sm = *reinterpret_cast<LatSmem<TIn> *>(smem_raw);
     const int tid = threadIdx.x;
@@ -303,8 +304,13 @@ cudaError_t launch_l(const ScanParams &p, cudaStream_t stream) {
     auto kern = scan_latency_kernel<TIn, HAS_H0>;
     cudaError_t e = ensure_smem(reinterpret_cast<const void *>(kern), smem);
     if (e != cudaSuccess) return e;
-    kern<<<static_cast<unsigned>(items), kLThreads, smem, stream>>>(p, cblocks);
-    e = cudaGetLastError();
+    if constexpr (HAS_H0) {
+        // a query's prefill, usually behind the retrieval of its row
+        e = launch_dependent(kern, dim3(static_cast<unsigned>(items)), dim3(kLThreads), smem, stream, p, cblocks);
+    } else {
+        kern<<<static_cast<unsigned>(items), kLThreads, smem, stream>>>(p, cblocks);
+        e = cudaGetLastError();
+    }
     if (e == cudaSuccess) count_launches(1);
     return e;
 }
