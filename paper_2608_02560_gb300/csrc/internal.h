@@ -76,8 +76,9 @@ cudaError_t ensure_smem(const void *kernel, int bytes);
 // Launch a kernel that opens with grid_dependency_wait(): its CTAs may become resident while
 // the stream's previous kernel still runs (programmatic stream serialization), which hides the
 // launch latency between the short kernels of the query path (retrieval, merge, prefill). Only
-// the tensor-core retrieval lets its merge in early: the shared-row kernel ran 4 us longer with
-// the merge's CTAs waiting beside it. One query, 2,000 x 384 keys, 24 x 32 tokens: 21.7 -> 18.3 us
+// the tensor-core retrieval of up to 32 queries lets its merge in early: the shared-row kernel
+// ran 4 us longer with the merge's CTAs waiting beside it, the tensor-core one of 64 to 128
+// queries 3 us. One query, 2,000 x 384 keys, 24 x 32 tokens: 21.7 -> 18.3 us
 // a pass; 256 queries, 100,000 x 768: 316.8 -> 313.9; top-3 of 23 fp32 queries 72.5 -> 69.5.
 template <class... KArgs, class... Args>
 cudaError_t launch_dependent(void (*kern)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t stream,

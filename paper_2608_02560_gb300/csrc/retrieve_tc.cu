@@ -42,8 +42,9 @@ constexpr int kBM = 128;          // queries per MMA (one half)
 constexpr int kBN = 256;          // key rows per tile at most (a multiple of 32)
 constexpr int kBK = 64;           // dim per k-block (128 bytes of fp16/bf16)
 constexpr int kMinRows = 64;      // and at least
-// Keys in flight per CTA: more of them queue in the memory system (192 KB: 1M x 768 keys 220
-// instead of 215 us; 128 KB of full tiles: 1M x 1024 286 instead of 284), less starve short tiles.
+// Keys in flight per CTA: more of them queue in the memory system (one query, 192 KB: 1M x 768
+// keys 220 instead of 215 us; 128 KB of full tiles: 1M x 1024 286 instead of 284), less starve
+// short tiles.
 constexpr uint32_t kKeyBytes = 112 * 1024;
 constexpr int kMaxStages = kKeyBytes / (kMinRows * kBK * 2);
 constexpr int kTopkStride = 8;    // keys per (CTA, query) in the top-k workspace
@@ -216,7 +217,7 @@ __global__ void __launch_bounds__(kThreads, 1)
                        const __grid_constant__ CUtensorMap tmap_k, int64_t M, int dim,
                        int n_queries, int q0, int nq, int a_rows, Ring ring, bool bf16,
                        unsigned long long *__restrict__ partial) {
-    grid_dependency_launch();   // the merge of the partial keys
+    if (n_queries <= kFewQueries) grid_dependency_launch();   // the merge of the partial keys
     extern __shared__ __align__(1024) uint8_t smem_raw[];
     Smem &sm = *reinterpret_cast<Smem *>(
         (reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~static_cast<uintptr_t>(1023));
@@ -410,7 +411,6 @@ __global__ void __launch_bounds__(kPairThreads, 1)
                             int q0, int nq, int bn, bool bf16, unsigned long long *__restrict__ partial) {
     using Sm = PairSmem<LIST>;
     constexpr int S = Sm::kStages;
-    grid_dependency_launch();   // the merge of the partial keys
     extern __shared__ __align__(1024) uint8_t smem_raw[];
     Sm &sm = *reinterpret_cast<Sm *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~static_cast<uintptr_t>(1023));
     const int warp = threadIdx.x >> 5;

@@ -502,7 +502,7 @@ __device__ __forceinline__ void scan_tile_direct(const unsigned char *st, const 
                 yv[j] = lo + hi;
             }
         }
-        if (C::HAS_Y && live) {
+        if constexpr (C::HAS_Y) {
             if (y_dtype == PRECOG_F32) {
                 float *dst = static_cast<float *>(yrow) + t * y_stride;
                 if constexpr (CPT == 2) {
@@ -1199,7 +1199,7 @@ __global__ void __launch_bounds__(C::LB_THREADS, C::LB_BLOCKS)
         } else if constexpr (C::RESCALED) {
             scan_tile_rescaled<C>(st, lay, reinterpret_cast<const float *>(st + (C::CONV ? lay.bf : lay.bs)), DS, dl, 0,
                                   ntok, h, Lw, kk, wmask, tot);
-        } else {
+        } else if (C::TRAJ || live) {   // (the branch around the loop: in it, it kept tokens apart)
             scan_tile_direct<C>(st, lay, DS, dl, ntok, h, kpow, kgen, live, yrow, p.y_dtype, y_stride, p, tcur,
                                 len - k * TILE, p.layer0 + layer, d0 + dl, tot);
         }
@@ -1261,9 +1261,13 @@ bool few_channels(const ScanParams &p) {
     return static_cast<int64_t>(p.n_layers) * p.n_chunks * p.D < static_cast<int64_t>(device_sm_count()) * kMaxSlice;
 }
 
-// At least six chunks of 256 channels per SM.
-bool many_channels(const ScanParams &p) {
-    return static_cast<int64_t>(p.n_layers) * p.n_chunks * p.D >= 6 * static_cast<int64_t>(device_sm_count()) * kMaxSlice;
+// Whether six CTAs per SM of four channels per thread take a launch in fewer rounds (counted in
+// CTAs per SM) than four of two channels per thread, whose tokens cost 7 % more.
+bool fits_quads(const ScanParams &p) {
+    const int64_t items = (static_cast<int64_t>(p.n_layers) * p.n_chunks * p.D + kMaxSlice - 1) / kMaxSlice;
+    const int64_t sms = device_sm_count();
+    const int64_t quads = (items + 6 * sms - 1) / (6 * sms) * 6, pairs = (items + 4 * sms - 1) / (4 * sms) * 4;
+    return 100 * quads <= 107 * pairs;
 }
 
 template <class C>
@@ -1363,12 +1367,12 @@ template <typename TIn, bool HAS_Y, bool HAS_H0, int MODE, int TRAJ = kTrajNone>
 cudaError_t launch_t(const ScanParams &p, cudaStream_t stream) {
     if constexpr (TRAJ != kTrajNone) {
         // power form: the rescaled or (short strides) the direct update, in the fp32 shape for
-        // any input but for wide strides over many 16-bit chunks, which are captures but for a
-        // few stores (stride 1000, 4 x 1000 x 1000 tokens: 1076 us, 1088 in the fp32 shape;
-        // stride 100, 4 x 250 x 750: 374, 345)
+        // any input but for wide strides of 16-bit chunks that fill rounds of the captures' shape
+        // (in that shape and in the fp32 one, us: stride 216, 4 x 208 x 2611 tokens 837, 882;
+        // stride 1000, 4 x 1000 x 750 1076, 1088; stride 100, 4 x 250 x 750 374, 345)
         if constexpr (MODE == kPower) {
             if constexpr (TRAJ == kTrajRescaled && !std::is_same<TIn, float>::value)
-                if (p.traj_stride >= 256 && many_channels(p))
+                if (p.traj_stride >= 64 && fits_quads(p))
                     return p.D % 256 == 0 && p.D % 512 != 0
                                ? launch_cfg<Cfg<TIn, false, false, kPower, PRECOG_RESCALED_CPT, PRECOG_RESCALED_TILE,
                                                 PRECOG_RESCALED_STAGES, PRECOG_RESCALED_MINB, TRAJ, kWideSlice, 256>>(p, stream)
@@ -1424,8 +1428,12 @@ cudaError_t launch_t(const ScanParams &p, cudaStream_t stream) {
             // 1000 chunks x 500 tokens fp32 1524 -> 1070 us, bf16 1096 -> 1032, with readout
             // 2126 -> 1419 and 1721 -> 1443. A readout launch that does not fill the SMs keeps
             // the deeper ring and the registers (24 x 3 x 500 bf16: 93 us, 102).
-            if constexpr (HAS_Y)
-                if (few_channels(p)) return launch_cfg<Cfg<TIn, HAS_Y, HAS_H0, MODE, 2, 16, 4, 3>>(p, stream);
+            if constexpr (HAS_Y) {
+                if (few_channels(p))
+                    return p.D % 256 == 0
+                               ? launch_cfg<Cfg<TIn, HAS_Y, HAS_H0, MODE, 2, 16, 4, 3, kTrajNone, kMaxSlice, 256>>(p, stream)
+                               : launch_cfg<Cfg<TIn, HAS_Y, HAS_H0, MODE, 2, 16, 4, 3>>(p, stream);
+            }
             if (p.D % 256 == 0)
                 return launch_cfg<Cfg<TIn, HAS_Y, HAS_H0, MODE, 2, 16, 2, 4, kTrajNone, kMaxSlice, 256>>(p, stream);
             return launch_cfg<Cfg<TIn, HAS_Y, HAS_H0, MODE, 2, 16, 2, 4>>(p, stream);
