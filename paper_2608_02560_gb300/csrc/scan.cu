@@ -94,7 +94,7 @@ struct Cfg {
     static constexpr bool SPLIT = SPLIT_;
     // 256-channel slices that stand in for 512-channel ones: the power statement is verified
     // for the 512 channels together, as by those.
-    static constexpr bool WIDE_CHECK = MODE_ == kPower && CPT_ == 2 && (SPLIT_ || MINB_ == 4);
+    static constexpr bool WIDE_CHECK = MODE_ == kPower && CPT_ == 2 && (SPLIT_ || TRAJ_ != kTrajNone || MINB_ == 4);
     // Widest channel slice of one CTA. Each CTA stages its slice of every token row; a
     // slice narrower than the row turns the row into separate pieces, and HBM serves
     // short scattered pieces far below its streaming rate, so rows up to 512 channels
@@ -109,7 +109,7 @@ struct Cfg {
     static constexpr int TRAJ = TRAJ_;
     static constexpr int MODE = MODE_, CPT = CPT_, TILE = TILE_, STAGES = STAGES_;
     // trajectory states leave through shared memory (see store_trajectory)
-    static constexpr bool STAGED = TRAJ_ != kTrajNone && MODE_ == kPower && CPT_ == 2;
+    static constexpr bool STAGED = TRAJ_ != kTrajNone && MODE_ == kPower && CPT_ == 2 && MINB_ == 4;
     static constexpr bool CONV = !std::is_same<TIn_, float>::value;
     static constexpr int SZ = sizeof(TIn_);
     static constexpr bool RESCALED = MODE_ == kPower && !HAS_Y_ && TRAJ_ != kTrajDirect;
@@ -422,7 +422,7 @@ template <class C>
 __device__ __forceinline__ void scan_tile_direct(const unsigned char *st, const StageLayout &lay,
                                                  int DS, int dl, int ntok,
                                                  f2 (&h)[C::CPT][8], const float (&kpow)[C::CPT],
-                                                 const f2 (&kgen)[C::CPT][8], bool live, void *yrow,
+                                                 const f2 (&kgen)[C::CPT][8], void *yrow,
                                                  int y_dtype, int64_t y_stride,
                                                  const ScanParams &p, TrajCursor &tc,
                                                  int64_t tok_left, int traj_layer, int dglob,
@@ -531,7 +531,7 @@ __device__ __forceinline__ void scan_tile_direct(const unsigned char *st, const 
                                           (row + tc.first) * kN, h);
                 } else {
 #pragma unroll
-                    for (int j = 0; live && j < CPT; ++j)
+                    for (int j = 0; j < CPT; ++j)
                         store_state16(p.traj, p.traj_dtype, (row + dglob + j) * kN, h[j]);
                 }
                 ++tc.entry;
@@ -1199,8 +1199,8 @@ __global__ void __launch_bounds__(C::LB_THREADS, C::LB_BLOCKS)
         } else if constexpr (C::RESCALED) {
             scan_tile_rescaled<C>(st, lay, reinterpret_cast<const float *>(st + (C::CONV ? lay.bf : lay.bs)), DS, dl, 0,
                                   ntok, h, Lw, kk, wmask, tot);
-        } else if (C::TRAJ || live) {   // (the branch around the loop: in it, it kept tokens apart)
-            scan_tile_direct<C>(st, lay, DS, dl, ntok, h, kpow, kgen, live, yrow, p.y_dtype, y_stride, p, tcur,
+        } else if (C::STAGED || live) {   // (the branch around the loop: in it, it kept tokens apart)
+            scan_tile_direct<C>(st, lay, DS, dl, ntok, h, kpow, kgen, yrow, p.y_dtype, y_stride, p, tcur,
                                 len - k * TILE, p.layer0 + layer, d0 + dl, tot);
         }
         if (C::HAS_Y) {
@@ -1378,6 +1378,9 @@ cudaError_t launch_t(const ScanParams &p, cudaStream_t stream) {
                                                 PRECOG_RESCALED_STAGES, PRECOG_RESCALED_MINB, TRAJ, kWideSlice, 256>>(p, stream)
                                : launch_cfg<Cfg<TIn, false, false, kPower, PRECOG_RESCALED_CPT, PRECOG_RESCALED_TILE,
                                                 PRECOG_RESCALED_STAGES, PRECOG_RESCALED_MINB, TRAJ, kWideSlice>>(p, stream);
+            // (launches that do not fill the SMs store plainly: each staged state adds to the
+            // chain of a lone warp, 24 x 1 x 250 x 64, every state: 57 us, 71)
+            if (few_channels(p)) return launch_cfg<Cfg<TIn, false, false, MODE, 2, 16, 2, 5, TRAJ, kMaxSlice>>(p, stream);
             return launch_pairs<TIn, false, false, TRAJ>(p, stream);
         } else {
             if (p.D % 256 == 0)
