@@ -7,8 +7,9 @@
 // each) and of B (and C) are staged into shared memory TILE tokens at a time
 // by the TMA engine, completing on an mbarrier, in a STAGES-deep ring, so the
 // time loop only reads shared memory: a whole-row slice is one contiguous 1-D
-// bulk copy per tensor; a narrower slice (rows wider than 512 channels) is one
-// tiled tensor-map copy of TILE rows per tensor.
+// bulk copy per tensor; a narrower slice (wide rows) is one tiled tensor-map
+// copy of TILE rows per tensor. Captures with few work items share a chunk's
+// tokens among the CTAs of a cluster (see combine).
 //
 // Per token and channel the recurrence is, for the 16 state indices n,
 //   h[n] <- alpha_n * h[n] + (dt * x) * B[n],   alpha_n = exp(dt * A[d, n]).
@@ -1388,22 +1389,25 @@ cudaError_t launch_t(const ScanParams &p, cudaStream_t stream) {
             return launch_cfg<Cfg<TIn, false, false, MODE, 2, 16, 4, 3, kTrajDirect>>(p, stream);
         }
     } else if constexpr (MODE == kPower && !HAS_Y) {
-        // the corpus encode of 256- and 512-channel slices (the paper's layer width, the
-        // ragged and wide workloads' slices) gets the slice fixed at compile time
-        if constexpr (std::is_same<TIn, float>::value) return launch_pairs<TIn, HAS_Y, HAS_H0, kTrajNone>(p, stream);
-        if constexpr (!HAS_H0) {
-            const int ds = pick_slice(p.D, kWideSlice);
-            if (ds == 256 && p.D % 256 == 0)
-                return launch_cfg<Cfg<TIn, false, false, MODE, PRECOG_RESCALED_CPT, PRECOG_RESCALED_TILE,
-                                      PRECOG_RESCALED_STAGES, PRECOG_RESCALED_MINB, kTrajNone, kWideSlice, 256>>(
-                    p, stream);
-            if (ds == 512)
-                return launch_cfg<Cfg<TIn, false, false, MODE, PRECOG_RESCALED_CPT, PRECOG_RESCALED_TILE,
-                                      PRECOG_RESCALED_STAGES, PRECOG_RESCALED_MINB, kTrajNone, kWideSlice, 512>>(
-                    p, stream);
+        if constexpr (std::is_same<TIn, float>::value) {
+            return launch_pairs<TIn, HAS_Y, HAS_H0, kTrajNone>(p, stream);
+        } else {
+            // the corpus encode of 256- and 512-channel slices (the paper's layer width, the
+            // ragged and wide workloads' slices) gets the slice fixed at compile time
+            if constexpr (!HAS_H0) {
+                const int ds = pick_slice(p.D, kWideSlice);
+                if (ds == 256 && p.D % 256 == 0)
+                    return launch_cfg<Cfg<TIn, false, false, MODE, PRECOG_RESCALED_CPT, PRECOG_RESCALED_TILE,
+                                          PRECOG_RESCALED_STAGES, PRECOG_RESCALED_MINB, kTrajNone, kWideSlice, 256>>(
+                        p, stream);
+                if (ds == 512)
+                    return launch_cfg<Cfg<TIn, false, false, MODE, PRECOG_RESCALED_CPT, PRECOG_RESCALED_TILE,
+                                          PRECOG_RESCALED_STAGES, PRECOG_RESCALED_MINB, kTrajNone, kWideSlice, 512>>(
+                        p, stream);
+            }
+            return launch_cfg<Cfg<TIn, HAS_Y, HAS_H0, MODE, PRECOG_RESCALED_CPT, PRECOG_RESCALED_TILE,
+                                  PRECOG_RESCALED_STAGES, PRECOG_RESCALED_MINB, kTrajNone, kWideSlice>>(p, stream);
         }
-        return launch_cfg<Cfg<TIn, HAS_Y, HAS_H0, MODE, PRECOG_RESCALED_CPT, PRECOG_RESCALED_TILE,
-                              PRECOG_RESCALED_STAGES, PRECOG_RESCALED_MINB, kTrajNone, kWideSlice>>(p, stream);
     } else {
         if constexpr (MODE == kPower) {
             // Fewer work items than SMs (a single query's prefill: one CTA per layer) is a
@@ -1413,17 +1417,22 @@ cudaError_t launch_t(const ScanParams &p, cudaStream_t stream) {
                 if (scan_latency_eligible(p)) return launch_scan_latency(p, stream);
                 return launch_cfg<Cfg<TIn, HAS_Y, HAS_H0, MODE, 2, 16, 2, 3>>(p, stream);
             }
-            if constexpr (std::is_same<TIn, float>::value) return launch_pairs<TIn, HAS_Y, HAS_H0, kTrajNone>(p, stream);
-            // 16-bit rows: 256- and 512-channel slices fixed at compile time
-            const int ds = pick_slice(p.D, kWideSlice);
-            if (ds == 256 && p.D % 256 == 0)
+            if constexpr (std::is_same<TIn, float>::value) {
+                return launch_pairs<TIn, HAS_Y, HAS_H0, kTrajNone>(p, stream);
+            } else {
+                // 16-bit rows: 256- and 512-channel slices fixed at compile time
+                const int ds = pick_slice(p.D, kWideSlice);
+                if (ds == 256 && p.D % 256 == 0)
+                    return launch_cfg<Cfg<TIn, HAS_Y, HAS_H0, MODE, PRECOG_DIRECT_CPT, PRECOG_DIRECT_TILE,
+                                          PRECOG_DIRECT_STAGES, PRECOG_DIRECT_MINB, kTrajNone, kWideSlice, 256>>(
+                        p, stream);
+                if (ds == 512)
+                    return launch_cfg<Cfg<TIn, HAS_Y, HAS_H0, MODE, PRECOG_DIRECT_CPT, PRECOG_DIRECT_TILE,
+                                          PRECOG_DIRECT_STAGES, PRECOG_DIRECT_MINB, kTrajNone, kWideSlice, 512>>(
+                        p, stream);
                 return launch_cfg<Cfg<TIn, HAS_Y, HAS_H0, MODE, PRECOG_DIRECT_CPT, PRECOG_DIRECT_TILE,
-                                      PRECOG_DIRECT_STAGES, PRECOG_DIRECT_MINB, kTrajNone, kWideSlice, 256>>(p, stream);
-            if (ds == 512)
-                return launch_cfg<Cfg<TIn, HAS_Y, HAS_H0, MODE, PRECOG_DIRECT_CPT, PRECOG_DIRECT_TILE,
-                                      PRECOG_DIRECT_STAGES, PRECOG_DIRECT_MINB, kTrajNone, kWideSlice, 512>>(p, stream);
-            return launch_cfg<Cfg<TIn, HAS_Y, HAS_H0, MODE, PRECOG_DIRECT_CPT, PRECOG_DIRECT_TILE,
-                                  PRECOG_DIRECT_STAGES, PRECOG_DIRECT_MINB, kTrajNone, kWideSlice>>(p, stream);
+                                      PRECOG_DIRECT_STAGES, PRECOG_DIRECT_MINB, kTrajNone, kWideSlice>>(p, stream);
+            }
         } else {
             // general A keeps 16 exponent coefficients per channel: 2 channels per thread. Two
             // stages and 128 registers let four CTAs share an SM's SFU (its bound: 16
