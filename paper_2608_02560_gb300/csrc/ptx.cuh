@@ -170,11 +170,12 @@ __device__ __forceinline__ uint32_t cluster_ctarank() {
     asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
     return r;
 }
-// Every thread of both CTAs; release/acquire orders shared-memory writes (barrier
-// initialisation included) before the peer's later accesses.
+// Every thread of the cluster's CTAs; release/acquire orders shared-memory writes (barrier
+// initialisation included) before a peer's later accesses. Not the .aligned forms: those need
+// the warp's threads converged, and callers come here from code that they leave one by one
+// (a thread without channels, a single producer lane).
 __device__ __forceinline__ void cluster_sync_all() {
-    asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" :::
-                     "memory");
+    asm volatile("barrier.cluster.arrive.release;\n\tbarrier.cluster.wait.acquire;" ::: "memory");
 }
 // The shared::cluster address of the object at `p`'s offset in the CTA of rank `rank`.
 __device__ __forceinline__ uint32_t mapa_shared(const void *p, uint32_t rank) {

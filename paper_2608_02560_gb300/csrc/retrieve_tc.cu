@@ -546,6 +546,7 @@ __global__ void __launch_bounds__(kPairThreads, 1)
     // neither CTA leaves (or frees tensor memory) while the other may still reach into it
     cluster_sync_all();
     if (warp == 1) {
+        __syncwarp();   // the barrier leaves the warp's convergence open, the release asks for it
         tc_fence_after();
         tmem_dealloc_pair(tmem, kTmemCols);
     }

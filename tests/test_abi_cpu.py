@@ -241,3 +241,13 @@ def test_extension_calls_reject_bad_arguments(lib):
     n = lib.precog_retrieve_noalloc
     assert n(FAKE, 2, 100, 768, FAKE, -1, FAKE, FAKE, None) == 1
     assert n(FAKE, 2, -1, 768, FAKE, 1, FAKE, FAKE, None) == 1
+
+
+def test_cluster_barrier_takes_diverged_warps():
+    """The cluster barrier follows branches and loops that a warp's threads leave one by one, so
+    neither half of it may be the .aligned form, which is undefined unless the warp has
+    converged. Nothing at run time shows the difference: the instructions are read instead."""
+    text = open(os.path.join(ROOT, "paper_2608_02560_gb300", "csrc", "ptx.cuh")).read()
+    forms = re.findall(r"barrier\.cluster\.(?:arrive|wait)[.a-z]*", text)
+    assert {f.split(".")[2] for f in forms} == {"arrive", "wait"}
+    assert not [f for f in forms if "aligned" in f]
