@@ -270,6 +270,15 @@ __device__ __forceinline__ float ex2(float x) {
     return y;
 }
 
+// v * 2^e + sum: beyond kExp2Near 2^e goes in three factors, so that a zero or tiny v does not
+// meet an infinite one. (2^e below fp32's range counts as zero.)
+constexpr float kExp2Near = 126.f;
+__device__ __forceinline__ float fma_exp2(float v, float e, float sum) {
+    if (!(e > kExp2Near)) return fmaf(ex2(e), v, sum);
+    const float f = ex2(fminf(e, 3.f * kExp2Near) * (1.f / 3.f));
+    return fmaf(v * f * f, f, sum);
+}
+
 // ---- packed fp32x2 (one instruction, two IEEE fp32 lanes, round to nearest) ----
 using f2 = unsigned long long;
 

@@ -20,6 +20,7 @@
 //              and a power chain per (t, d); with a readout y the state is
 //              updated directly, without one it is accumulated rescaled
 //              (see scan_tile_rescaled), which drops the per-n decay multiply.
+#include <cfloat>
 #include <type_traits>
 
 #include "../../include/precog.h"
@@ -808,7 +809,11 @@ __device__ __forceinline__ void scan_tile_rescaled(const unsigned char *st, cons
 // Every CTA leaves its h_s and its sum of dt in its shared memory; the cluster's threads
 // share the (channel, 4 states) sums, each from the last segment back, and write the states. Each
 // segment's sum is relative to its own tokens, so a factor far below 1 belongs to a state
-// that no longer matters and the rounding of its exponent is scaled down with it.
+// that no longer matters and the rounding of its exponent is scaled down with it. Modes that grow
+// (a negative sum of dt, or A > 0) may have factors beyond fp32's range where the state is zero or
+// small enough to stay finite; those sums are formed again with fma_exp2. (Redoing the rare
+// sum costs the usual one nothing, 24 layers x 3 x 500 tokens 30.7 us; a choice per factor
+// inside it took 31.9 to 34.8 us.)
 struct SplitSmem {
     int32_t dead;      // this CTA gave up on a wait
     int32_t pad[31];
@@ -843,15 +848,33 @@ __device__ __forceinline__ void combine(unsigned char *buf, const ScanParams &p,
         const int q = i / DS, ch = i % DS;
         if (d0 + ch >= p.D) continue;
         const float4 a = *reinterpret_cast<const float4 *>(Al + static_cast<int64_t>(d0 + ch) * kN + 4 * q);
-        const float c[4] = {a.x * kLog2e, a.y * kLog2e, a.z * kLog2e, a.w * kLog2e};
+        // (finite, so that a mode without memory, A = -inf, times no dt is no decay)
+        const auto coeff = [](float x) { return fminf(fmaxf(x * kLog2e, -FLT_MAX), FLT_MAX); };
+        const float c[4] = {coeff(a.x), coeff(a.y), coeff(a.z), coeff(a.w)};
         float after = 0.f;   // dt summed over the segments after the current one
+        float most = 0.f, least = 0.f;
         float sum[4] = {0.f, 0.f, 0.f, 0.f};
         for (int s = segs - 1; s >= 0; --s) {
             const float4 v = ld_cluster_f4(mapa_shared(&hs[q * DS + ch], s));
             const float hv[4] = {v.x, v.y, v.z, v.w};
+            most = fmaxf(most, after);
+            least = fminf(least, after);
 #pragma unroll
             for (int k = 0; k < 4; ++k) sum[k] = fmaf(ex2(c[k] * after), hv[k], sum[k]);
             after += __uint_as_float(ld_cluster_u32(mapa_shared(&ts[ch], s)));
+        }
+        const float chigh = fmaxf(fmaxf(c[0], c[1]), fmaxf(c[2], c[3])), clow = fminf(fminf(c[0], c[1]), fminf(c[2], c[3]));
+        if (fmaxf(fmaxf(chigh * most, chigh * least), fmaxf(clow * most, clow * least)) > kExp2Near) {
+            // once more (the usual sum above has no branches)
+            after = sum[0] = sum[1] = sum[2] = sum[3] = 0.f;
+#pragma unroll 1
+            for (int s = segs - 1; s >= 0; --s) {
+                const float4 v = ld_cluster_f4(mapa_shared(&hs[q * DS + ch], s));
+                const float hv[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+                for (int k = 0; k < 4; ++k) sum[k] = fma_exp2(hv[k], c[k] * after, sum[k]);
+                after += __uint_as_float(ld_cluster_u32(mapa_shared(&ts[ch], s)));
+            }
         }
         const int64_t off = ((chunk * p.L_out + p.layer0 + layer) * static_cast<int64_t>(p.D) + d0 + ch) * kN + 4 * q;
         if (p.state_dtype == PRECOG_F32) {

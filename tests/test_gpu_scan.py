@@ -623,3 +623,38 @@ def test_split_chunks(cuda_device, kind, power, L, D, lens):
         assert st != 0 and bits & pg.PRECOG_DEV_BAD_OFFSETS
         assert (out[1:3] == 7.0).all()
         assert torch.equal(out[[0, 3, 4]], states[[0, 3, 4]])
+
+
+@pytest.mark.parametrize("kind", ["bf16", "f32"])
+@pytest.mark.parametrize("power", [True, False])
+@pytest.mark.parametrize("T", [512, 100])
+@pytest.mark.parametrize("first", [0.0, 1e-36])
+def test_split_growing_modes(cuda_device, kind, power, T, first):
+    """Modes that grow by more than 2^128 over the shares (net negative dt, or positive entries of A)
+    from an early state that is exactly zero or tiny: the combination is finite where the state
+    is, as the unsplit scan. x is `first` in the first 8 tokens, zero up to the last 32. Relative
+    to each state index's largest value: the usual tolerance, and e^E after E nats, whose
+    exponent is a sum of up to a share's tokens and the shares."""
+    import torch
+    dtype = torch.float32 if kind == "f32" else torch.bfloat16
+    x, dt, _, B, _ = synth.host_scan_inputs(T, 64, 16, seed=5 * T)
+    rng = np.random.default_rng(T)
+    dt = (10.24 / T * rng.uniform(0.5, 1.5, size=dt.shape)).astype(np.float32)   # sums to 10.24
+    n = np.arange(1, 17, dtype=np.float32)
+    A = np.tile(-n if power else n * (-1.0) ** n, (64, 1)).astype(np.float32)
+    x[8:-32] = 0
+    x[:8] *= np.float32(first)
+    if power:
+        dt = -dt
+    else:
+        A[:, 4] = -np.inf                       # a mode without memory
+    xs, dts, Bs = (_t(a, cuda_device, dtype) for a in (x, dt, B))
+    off = np.array([0, T], np.int64)
+    states, _ = _encode(cuda_device, xs, dts, Bs, _t(A, cuda_device), _t(off, cuda_device, torch.int64), power=power)
+    got = to_np(states[0, 0])
+    ref, _ = oracle.scan(to_np(xs), to_np(dts), A, to_np(Bs), off)
+    assert np.all(np.isfinite(got)) and np.abs(ref).max() < 3e38
+    nats = np.where(np.isinf(A), 0, np.abs(A)).max(axis=0) * np.abs(to_np(dts)).sum(axis=0).max()
+    tol = TOL_F32 if kind == "f32" else TOL_BF16
+    err = np.abs(got - ref[0]).max(axis=0) / np.abs(ref[0]).max(axis=0)
+    assert np.all(err < tol + nats * (T / 4 + 16 + 8) * 2.0 ** -24)
