@@ -178,11 +178,12 @@ __device__ __forceinline__ void cluster_sync_all() {
     asm volatile("barrier.cluster.arrive.release;\n\tbarrier.cluster.wait.acquire;" ::: "memory");
 }
 // The shared::cluster address of the object at `p`'s offset in the CTA of rank `rank`.
-__device__ __forceinline__ uint32_t mapa_shared(const void *p, uint32_t rank) {
+__device__ __forceinline__ uint32_t mapa_shared(uint32_t own, uint32_t rank) {
     uint32_t r;
-    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(smem_u32(p)), "r"(rank));
+    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(own), "r"(rank));
     return r;
 }
+__device__ __forceinline__ uint32_t mapa_shared(const void *p, uint32_t rank) { return mapa_shared(smem_u32(p), rank); }
 // Loads from the shared memory of a CTA of the cluster (address from mapa_shared).
 __device__ __forceinline__ uint32_t ld_cluster_u32(uint32_t addr) {
     uint32_t v;

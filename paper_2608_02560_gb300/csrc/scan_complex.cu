@@ -22,6 +22,7 @@
 // of the weights and two real FMAs per state index, see renormalise_c; harmonic form:
 // the rotation tree and one exponential per index, see renormalise_h). Other A, and
 // fp32 inputs, keep the per-index form.
+#include <cfloat>
 #include <type_traits>
 
 #include "../../include/precog.h"
@@ -351,6 +352,7 @@ constexpr int block_channels() { return HAS_Y ? 128 : 256; }
 // own final state (from zero) decayed by the tokens after it, h = sum_s exp(A * dt_s) h_s with
 // dt_s the dt summed over the segments after s. The decay's phase A_im * dt_s may be many
 // turns, so dt is summed to twice fp32 precision and the phase formed as a two-float product.
+// As there, sums with factors beyond fp32's range are formed again with fma_exp2.
 struct DtSum {
     float hi, lo;
     __device__ __forceinline__ void add(float v) {   // Knuth's two-sum
@@ -366,6 +368,58 @@ struct SplitState {
     alignas(16) float4 h[kN / 2][CB];   // states 2i, 2i+1 of a channel as (re, im, re, im)
     float2 dt[CB];
 };
+
+// The segments' sum of h_s e^(A dt_s) for two states of a channel, (re, im, re, im): h_own and
+// dt_own are this CTA's shared-memory addresses of them and of the dt sum, c0, c1 the states'
+// A_re log2 e and ai their A_im. The first form also notes the largest and least dt_s; GROWS: the
+// factors' magnitudes may be beyond fp32's range.
+template <bool GROWS>
+__device__ __forceinline__ float4 sum_segments(uint32_t h_own, uint32_t dt_own, int segs, float c0, float c1, f2 ai,
+                                               float &most, float &least) {
+    const f2 ar = pack2(c0, c1);
+    DtSum after{0.f, 0.f};
+    f2 sr = 0, si = 0;
+    constexpr int kUnroll = GROWS ? 1 : 4;
+#pragma unroll kUnroll
+    for (int s = segs - 1; s >= 0; --s) {
+        const float4 v = ld_cluster_f4(mapa_shared(h_own, s));
+        const f2 vr = pack2(v.x, v.z), vi = pack2(v.y, v.w), dd = pack2(after.hi, after.hi);
+        float e0, e1;
+        unpack2(mul2(dd, ar), e0, e1);
+        const f2 th = mul2(dd, ai);
+        float t0, t1;
+        unpack2(th, t0, t1);
+        const f2 tl = fma2(pack2(after.lo, after.lo), ai, fma2(dd, ai, pack2(-t0, -t1)));
+        f2 sn, cs;
+        sincos_pair(th, tl, sn, cs);
+        float i0, i1;
+        unpack2(vi, i0, i1);
+        const f2 nvi = pack2(-i0, -i1);
+        if constexpr (GROWS) {
+            float r0, r1, s0, s1;
+            unpack2(fma2(cs, vr, mul2(sn, nvi)), r0, r1);
+            unpack2(sr, s0, s1);
+            sr = pack2(fma_exp2(r0, e0, s0), fma_exp2(r1, e1, s1));
+            unpack2(fma2(cs, vi, mul2(sn, vr)), r0, r1);
+            unpack2(si, s0, s1);
+            si = pack2(fma_exp2(r0, e0, s0), fma_exp2(r1, e1, s1));
+        } else {
+            most = fmaxf(most, after.hi);
+            least = fminf(least, after.hi);
+            const f2 mag = pack2(ex2(e0), ex2(e1));
+            const f2 fr = mul2(mag, cs), fi = mul2(mag, sn);
+            sr = fma2(fr, vr, fma2(fi, nvi, sr));
+            si = fma2(fr, vi, fma2(fi, vr, si));
+        }
+        const uint32_t at = mapa_shared(dt_own, s);
+        after.add(__uint_as_float(ld_cluster_u32(at)));
+        after.lo += __uint_as_float(ld_cluster_u32(at + 4));
+    }
+    float r0, r1, i0, i1;
+    unpack2(sr, r0, r1);
+    unpack2(si, i0, i1);
+    return make_float4(r0, i0, r1, i1);
+}
 
 template <int CB>
 __device__ __forceinline__ void combine(unsigned char *buf, const ScanParams &p, bool dead, bool live, int W,
@@ -387,38 +441,19 @@ __device__ __forceinline__ void combine(unsigned char *buf, const ScanParams &p,
         const int q = i / W, ch = i % W;
         const int64_t row = static_cast<int64_t>(layer) * p.D + d0 + ch;
         const float4 a = reinterpret_cast<const float4 *>(p.A)[row * (kN / 2) + q];
-        const f2 ar = pack2(a.x * kLog2e, a.z * kLog2e), ai = pack2(a.y, a.w);
-        DtSum after{0.f, 0.f};
-        f2 sr = 0, si = 0;
-        for (int s = segs - 1; s >= 0; --s) {
-            const float4 v = ld_cluster_f4(mapa_shared(&sm.h[q][ch], s));
-            const f2 vr = pack2(v.x, v.z), vi = pack2(v.y, v.w), dd = pack2(after.hi, after.hi);
-            float e0, e1;
-            unpack2(mul2(dd, ar), e0, e1);
-            const f2 mag = pack2(ex2(e0), ex2(e1));
-            const f2 th = mul2(dd, ai);
-            float t0, t1;
-            unpack2(th, t0, t1);
-            const f2 tl = fma2(pack2(after.lo, after.lo), ai, fma2(dd, ai, pack2(-t0, -t1)));
-            f2 sn, cs;
-            sincos_pair(th, tl, sn, cs);
-            const f2 fr = mul2(mag, cs), fi = mul2(mag, sn);
-            float i0, i1;
-            unpack2(vi, i0, i1);
-            sr = fma2(fr, vr, fma2(fi, pack2(-i0, -i1), sr));
-            si = fma2(fr, vi, fma2(fi, vr, si));
-            const uint32_t at = mapa_shared(&sm.dt[ch], s);
-            after.add(__uint_as_float(ld_cluster_u32(at)));
-            after.lo += __uint_as_float(ld_cluster_u32(at + 4));
-        }
-        float r0, r1, i0, i1;
-        unpack2(sr, r0, r1);
-        unpack2(si, i0, i1);
+        // (finite, so that a mode without memory, an infinite A_re, times no dt is no decay)
+        const float c0 = fminf(fmaxf(a.x * kLog2e, -FLT_MAX), FLT_MAX), c1 = fminf(fmaxf(a.z * kLog2e, -FLT_MAX), FLT_MAX);
+        const f2 ai = pack2(a.y, a.w);
+        const uint32_t h_own = smem_u32(&sm.h[q][ch]), dt_own = smem_u32(&sm.dt[ch]);
+        float most = 0.f, least = 0.f;
+        float4 h = sum_segments<false>(h_own, dt_own, segs, c0, c1, ai, most, least);
+        if (fmaxf(fmaxf(c0 * most, c0 * least), fmaxf(c1 * most, c1 * least)) > kExp2Near)
+            h = sum_segments<true>(h_own, dt_own, segs, c0, c1, ai, most, least);
         const int64_t off = ((chunk * p.L_out + p.layer0 + layer) * static_cast<int64_t>(p.D) + d0 + ch) * kN + 2 * q;
         if (p.state_dtype == PRECOG_F32) {
-            *reinterpret_cast<float4 *>(static_cast<float *>(p.states) + 2 * off) = make_float4(r0, i0, r1, i1);
+            *reinterpret_cast<float4 *>(static_cast<float *>(p.states) + 2 * off) = h;
         } else {
-            const __nv_bfloat162 lo = __floats2bfloat162_rn(r0, i0), up = __floats2bfloat162_rn(r1, i1);
+            const __nv_bfloat162 lo = __floats2bfloat162_rn(h.x, h.y), up = __floats2bfloat162_rn(h.z, h.w);
             *reinterpret_cast<uint2 *>(static_cast<__nv_bfloat16 *>(p.states) + 2 * off) =
                 make_uint2(*reinterpret_cast<const uint32_t *>(&lo), *reinterpret_cast<const uint32_t *>(&up));
         }

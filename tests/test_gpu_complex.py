@@ -332,3 +332,47 @@ def test_complex_split_chunks(cuda_device, D, lens, form, in16):
         assert _cplx_err(hs[c], ref_h[c]) < max(tol, 1.25 * unsplit)
     half, _ = _encode(pg, cuda_device, x, dt, B, C, A, offsets, with_y=False, in_dtype=in_dtype, state_dtype="bf16")
     assert rel_err_stored(half.real, hs.real) < 1e-7 and rel_err_stored(half.imag, hs.imag) < 1e-7
+
+
+@pytest.mark.parametrize("in16", [False, True])
+@pytest.mark.parametrize("form", FORMS)
+@pytest.mark.parametrize("T", [512, 150])
+@pytest.mark.parametrize("first", [0.0, 1e-36])
+def test_complex_split_growing_modes(cuda_device, form, in16, T, first):
+    """Modes that grow by more than 2^128 over the shares (net negative dt) from an early state that is
+    exactly zero or tiny: the combination is finite where the state is. x is `first` in the first
+    8 tokens, zero up to the last 32. Relative to each state index's largest value: the usual
+    tolerance or the unsplit scan's error (state-only prefill from the zero state), and e^E after
+    E nats, whose exponent is a sum of up to a share's tokens and the shares."""
+    import torch
+    pg = _pg()
+    D = 64
+    in_dtype = torch.bfloat16 if in16 else None
+    rng = np.random.default_rng(T)
+    x, dt, _, B, C = synth.host_scan_inputs(T, D, 16, seed=T)
+    A = _complex_A(D, 16, 3, form)
+    x[8:-32] = 0
+    x[:8] *= np.float32(first)
+    # every channel's fastest mode grows by about 150 nats
+    dt = (-150.0 / T * rng.uniform(0.7, 1.3, size=dt.shape) / np.abs(A.real).max(axis=1)).astype(np.float32)
+    nats = (np.abs(A.real) * np.abs(dt).sum(axis=0)[:, None]).max(axis=0)
+    if form == "index":
+        A.real[:, 4] = np.inf                   # a mode without memory, as dt < 0
+        nats[4] = 0
+    if in16:
+        rnd = lambda a: torch.from_numpy(a).to(torch.bfloat16).float().numpy()
+        x, dt, B = rnd(x), rnd(dt), rnd(B)
+    off = np.array([0, T], np.int64)
+    hs, _ = _encode(pg, cuda_device, x, dt, B, C, A, off, with_y=False, in_dtype=in_dtype)
+    ref, _ = oracle.scan_complex(x, dt, A.real, A.imag, B, off)
+    assert np.abs(ref).max() < 3e38 and np.all(np.isfinite(hs))
+    pg_in = lambda a: _t(a, cuda_device, in_dtype)
+    one = torch.empty((1, 1, D, 16), dtype=torch.complex64, device=cuda_device)
+    pg.precog_prefill_from_state(
+        pg.scan_inputs(pg_in(x), pg_in(dt), pg_in(B), _t(A, cuda_device), a_kind=pg.PRECOG_A_COMPLEX), 1, T,
+        torch.zeros((1, 1, D, 16), dtype=torch.complex64, device=cuda_device),
+        torch.tensor([-1], device=cuda_device), state_out=one)
+    per_index = lambda h: np.abs(np.asarray(h, np.complex128) - ref[0]).max(axis=0) / np.abs(ref[0]).max(axis=0)
+    unsplit = per_index(one[0, 0].cpu().numpy())
+    assert np.all(per_index(hs[0]) < np.maximum(TOL_BF16 if in16 else TOL_F32, 1.25 * unsplit)
+                  + nats * (T / 4 + 32 + 8) * 2.0 ** -24)
