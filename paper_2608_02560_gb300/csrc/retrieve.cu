@@ -45,21 +45,31 @@ __device__ __forceinline__ unsigned long long make_key(float s, int64_t row) {
 template <typename T> struct Vec;
 template <> struct Vec<float> { static constexpr int n = 4; };
 
-template <typename T>
-__device__ __forceinline__ void widen(const uint4 &v, float (&f)[Vec<T>::n]) {
-    static_assert(std::is_same<T, float>::value, "fp32 keys only");
-    f[0] = __uint_as_float(v.x);
-    f[1] = __uint_as_float(v.y);
-    f[2] = __uint_as_float(v.z);
-    f[3] = __uint_as_float(v.w);
+// The products of one 16-byte vector of a row with a query's, and a lane's sum of them. Every
+// fp32 kernel sums a row in this order (a lane's vectors l, l+32, ... with even and odd elements
+// apart, then the lanes' sums over xor distances 16, 8, 4, 2, 1), so that a score does not depend
+// on the kernel that the number of queries or k selects.
+__device__ __forceinline__ void dot_step(f2 &acc, const ulonglong2 &x, const f2 (&q)[2]) {
+    acc = fma2(x.x, q[0], acc);
+    acc = fma2(x.y, q[1], acc);
+}
+__device__ __forceinline__ float dot_sum(f2 acc) {
+    float lo, hi;
+    unpack2(acc, lo, hi);
+    return lo + hi;
+}
+// Vector v of a row of floats (zeros where it is not to be read).
+__device__ __forceinline__ ulonglong2 load_vec(const float *row, int v, bool in) {
+    return in ? __ldg(reinterpret_cast<const ulonglong2 *>(row) + v) : make_ulonglong2(0ull, 0ull);
 }
 
 // partial[blockIdx.x * n_queries + q] = best key of this CTA for query q.
 // Lane l owns the 16-byte vectors l, l+32, ... of every row (VPL of them) and
 // holds the matching query values in registers; RIF rows are loaded before any
 // is used, so each lane keeps RIF*VPL 16-byte loads in flight.
+// Two vectors per lane keep four CTAs per SM (200,000 x 256 keys 37 us; 78 registers, three: 45).
 template <typename T, int QB, int VPL, int RIF>
-__global__ void __launch_bounds__(kThreads)
+__global__ void __launch_bounds__(kThreads, QB == 1 && VPL == 2 ? 4 : 1)
     gemv_top1_kernel(const T *__restrict__ index, int64_t M, int dim, const T *__restrict__ queries,
                      int n_queries, int q0, unsigned long long *__restrict__ partial) {
     constexpr int V = Vec<T>::n;
@@ -68,20 +78,15 @@ __global__ void __launch_bounds__(kThreads)
     const int lane = threadIdx.x & 31;
     const int warp = threadIdx.x >> 5;
     const int vecs = dim / V;
-    float qv[QB][VPL][V];
+    f2 qv[QB][VPL][2];
 #pragma unroll
     for (int qq = 0; qq < QB; ++qq)
 #pragma unroll
         for (int j = 0; j < VPL; ++j) {
             const int v = lane + 32 * j;
-            if (qq < nq && v < vecs) {
-                const uint4 raw =
-                    __ldg(reinterpret_cast<const uint4 *>(queries + static_cast<int64_t>(q0 + qq) * dim) + v);
-                widen<T>(raw, qv[qq][j]);
-            } else {
-#pragma unroll
-                for (int e = 0; e < V; ++e) qv[qq][j][e] = 0.f;
-            }
+            const ulonglong2 raw = load_vec(queries + static_cast<int64_t>(q0 + qq) * dim, v, qq < nq && v < vecs);
+            qv[qq][j][0] = raw.x;
+            qv[qq][j][1] = raw.y;
         }
     if (threadIdx.x < QB) best[threadIdx.x] = 0ull;
     __syncthreads();
@@ -93,35 +98,28 @@ __global__ void __launch_bounds__(kThreads)
     for (int qq = 0; qq < QB; ++qq) mykey[qq] = 0ull;
 
     for (int64_t r0 = gwarp * RIF; r0 < M; r0 += nwarps * RIF) {
-        uint4 raw[RIF][VPL];
+        ulonglong2 raw[RIF][VPL];
 #pragma unroll
         for (int r = 0; r < RIF; ++r)
 #pragma unroll
             for (int j = 0; j < VPL; ++j) {
                 const int v = lane + 32 * j;
                 const int64_t row = r0 + r;
-                raw[r][j] = (v < vecs && row < M)
-                                ? __ldg(reinterpret_cast<const uint4 *>(index + row * dim) + v)
-                                : make_uint4(0, 0, 0, 0);
+                raw[r][j] = load_vec(index + row * dim, v, v < vecs && row < M);
             }
 #pragma unroll
         for (int r = 0; r < RIF; ++r) {
-            float acc[QB];
+            f2 acc[QB];
 #pragma unroll
-            for (int qq = 0; qq < QB; ++qq) acc[qq] = 0.f;
+            for (int qq = 0; qq < QB; ++qq) acc[qq] = 0;
 #pragma unroll
-            for (int j = 0; j < VPL; ++j) {
-                float f[V];
-                widen<T>(raw[r][j], f);
+            for (int j = 0; j < VPL; ++j)
 #pragma unroll
-                for (int qq = 0; qq < QB; ++qq)
-#pragma unroll
-                    for (int e = 0; e < V; ++e) acc[qq] = fmaf(f[e], qv[qq][j][e], acc[qq]);
-            }
+                for (int qq = 0; qq < QB; ++qq) dot_step(acc[qq], raw[r][j], qv[qq][j]);
             const int64_t row = r0 + r;
 #pragma unroll
             for (int qq = 0; qq < QB; ++qq) {
-                float sc = acc[qq];
+                float sc = dot_sum(acc[qq]);
 #pragma unroll
                 for (int o = 16; o > 0; o >>= 1) sc += __shfl_xor_sync(0xffffffffu, sc, o);
                 if (row < M && !isnan(sc)) {
@@ -228,17 +226,13 @@ __global__ void __launch_bounds__(kThreads)
     const int lane = threadIdx.x & 31;
     const int warp = threadIdx.x >> 5;
     const int vecs = dim / V;
-    float qv[VPL][V];
+    f2 qv[VPL][2];
 #pragma unroll
     for (int j = 0; j < VPL; ++j) {
         const int v = lane + 32 * j;
-        if (v < vecs) {
-            const uint4 raw = __ldg(reinterpret_cast<const uint4 *>(queries + static_cast<int64_t>(q) * dim) + v);
-            widen<T>(raw, qv[j]);
-        } else {
-#pragma unroll
-            for (int e = 0; e < V; ++e) qv[j][e] = 0.f;
-        }
+        const ulonglong2 raw = load_vec(queries + static_cast<int64_t>(q) * dim, v, v < vecs);
+        qv[j][0] = raw.x;
+        qv[j][1] = raw.y;
     }
     unsigned long long l[kListK];
 #pragma unroll
@@ -246,27 +240,21 @@ __global__ void __launch_bounds__(kThreads)
     const int64_t gwarp = static_cast<int64_t>(blockIdx.x) * kWarps + warp;
     const int64_t nwarps = static_cast<int64_t>(gridDim.x) * kWarps;
     for (int64_t r0 = gwarp * RIF; r0 < M; r0 += nwarps * RIF) {
-        uint4 raw[RIF][VPL];
+        ulonglong2 raw[RIF][VPL];
 #pragma unroll
         for (int r = 0; r < RIF; ++r)
 #pragma unroll
             for (int j = 0; j < VPL; ++j) {
                 const int v = lane + 32 * j;
                 const int64_t row = r0 + r;
-                raw[r][j] = (v < vecs && row < M)
-                                ? __ldg(reinterpret_cast<const uint4 *>(index + row * dim) + v)
-                                : make_uint4(0, 0, 0, 0);
+                raw[r][j] = load_vec(index + row * dim, v, v < vecs && row < M);
             }
 #pragma unroll
         for (int r = 0; r < RIF; ++r) {
-            float acc = 0.f;
+            f2 sums = 0;
 #pragma unroll
-            for (int j = 0; j < VPL; ++j) {
-                float f[V];
-                widen<T>(raw[r][j], f);
-#pragma unroll
-                for (int e = 0; e < V; ++e) acc = fmaf(f[e], qv[j][e], acc);
-            }
+            for (int j = 0; j < VPL; ++j) dot_step(sums, raw[r][j], qv[j]);
+            float acc = dot_sum(sums);
 #pragma unroll
             for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
             const int64_t row = r0 + r;
@@ -493,17 +481,10 @@ __global__ void __launch_bounds__(kGemmThreads, 1)
                     const int v = lane + 32 * j;
                     const ulonglong2 x = v < vecs ? src[v] : make_ulonglong2(0ull, 0ull);
 #pragma unroll
-                    for (int i = 0; i < QW; ++i) {
-                        acc[i] = fma2(x.x, qv[i][j][0], acc[i]);
-                        acc[i] = fma2(x.y, qv[i][j][1], acc[i]);
-                    }
+                    for (int i = 0; i < QW; ++i) dot_step(acc[i], x, qv[i][j]);
                 }
 #pragma unroll
-                for (int i = 0; i < QW; ++i) {
-                    float lo, hi;
-                    unpack2(acc[i], lo, hi);
-                    a[r * QW + i] = lo + hi;
-                }
+                for (int i = 0; i < QW; ++i) a[r * QW + i] = dot_sum(acc[i]);
             }
             int o = 16;
 #pragma unroll
@@ -671,9 +652,10 @@ cudaError_t launch_gemv_topk(const RetrieveParams &p, cudaStream_t stream, int g
 
 // fp32 keys of up to kGemmMaxDim dims go to the shared-row kernel. A single query's pass does
 // up to 8 queries' arithmetic there, so it goes where that is faster (us, GEMV / shared rows):
-// top-1 over rows of more than 512 dims (300,000 x 768: 181 / 139; 200,000 x 256: 42 / 47; 384
-// and 512 dims within 2 %); top-k always (50,021 x 384, k = 3: 36 / 24) but for long lists over
-// 257 to 384 dims, where insertions stall its few warps (500,000 x 384, k = 8: 146 / 180).
+// top-1 over rows of more than 512 dims (300,000 x 768: 181 / 139; 200,000 x 256: 37 / 42;
+// 300,000 x 384: 71 / 82; 200,000 x 512: 63 / 63); top-k always (50,021 x 384, k = 3: 36 / 24) but
+// for long lists over 257 to 384 dims, where insertions stall its few warps (k = 8, 500,000 x
+// 384: 141 / 175; 50,021 x 384: 34 / 29).
 bool use_gemm(const RetrieveParams &p, bool topk, int k) {
     if (p.dim > kGemmMaxDim) return false;
     if (p.n_queries > 1) return true;

@@ -178,3 +178,28 @@ def test_f32_batches_share_rows(cuda_device, M, dim, Q):
             assert pg.precog_device_status()[0] == 0
             np.testing.assert_array_equal(i1.cpu().numpy(), idx[:, 0])
             np.testing.assert_array_equal(s1.cpu().numpy(), score[:, 0])
+
+
+@pytest.mark.parametrize("M,dim", [(3001, 64), (3001, 384), (3001, 512), (1500, 516), (1500, 1024), (900, 1280)])
+def test_fp32_scores_do_not_depend_on_the_call(cuda_device, M, dim):
+    """One query's score of a row is the same bit for bit alone or in a batch, and in a top-1 or a
+    top-k call, whichever kernel the sizes choose (fp32 keys: per-row kernels, the shared-row
+    kernel with 8, 4 or 2 queries per group), so near-tied rows rank the same everywhere."""
+    import torch
+    pg = _pg()
+    gen = torch.Generator(device=cuda_device).manual_seed(M + dim)
+    index = torch.randn((M, dim), generator=gen, device=cuda_device)
+    index[1::2] = index[::2][: M // 2] * (1 + 1e-7 * torch.randn((M // 2, 1), generator=gen, device=cuda_device))
+    queries = torch.randn((9, dim), generator=gen, device=cuda_device)
+    batch_i, batch_s = _topk(index, queries, 8)
+    for n in (1, 2, 9):
+        i1 = torch.empty(n, dtype=torch.int64, device=cuda_device)
+        s1 = torch.empty(n, dtype=torch.float32, device=cuda_device)
+        pg.precog_retrieve(index, queries[:n], i1, s1)
+        np.testing.assert_array_equal(s1.cpu().numpy(), batch_s[:n, 0])
+        np.testing.assert_array_equal(i1.cpu().numpy(), batch_i[:n, 0])
+        for k in (3, 8):
+            idx, score = _topk(index, queries[:n], k)
+            np.testing.assert_array_equal(score, batch_s[:n, :k])
+            np.testing.assert_array_equal(idx, batch_i[:n, :k])
+    assert pg.precog_device_status()[0] == 0
