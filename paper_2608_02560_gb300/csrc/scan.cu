@@ -1354,22 +1354,31 @@ cudaError_t launch_cfg(const ScanParams &p, cudaStream_t stream) {
     return e;
 }
 
-// CTAs per chunk of a capture (1: not split), a power of two up to the portable cluster size.
-// One CTA takes about 0.12 us per token whatever else runs, so a launch that leaves SMs without
-// a CTA or with one is as long as its chunks; split, a chunk of 24 layers x 3 x 500 tokens
-// takes 70 -> 27 us, 1 x 1 x 4096 517 -> 60, 24 x 6 x 500 70 -> 43, 24 x 9 x 500 73 -> 60
-// (bf16 power form; general A 60 -> 33, 448 -> 71, 60 -> 54, 93 -> 77). From 1.5 items per SM
-// on the unsplit launch fills the SMs (24 x 12 x 500: 72.5 against 76; general 93 against
-// 101), and below 80 tokens the combination costs what the shorter chains save.
+// CTAs per chunk of a capture (8 or 4; 1: not split). One CTA takes 0.09 (fp32) to 0.14 us per
+// token whatever else runs, so a launch that leaves SMs without a CTA or with one is as long as its
+// chunks. A split launch has `segs` times the CTAs, each with its ring, its rows of A and its
+// part of the combination, and with fp32 inputs only three of them fit an SM; so the chunks must
+// be the longer, the more CTAs an SM would get: at least kPerChannels tokens per 256
+// channels and kPerCta per CTA on an SM, and 80. us, unsplit / split as chosen (bf16 power):
+// 24 layers x 3 chunks x 500 tokens 70 / 27, 1 x 1 x 4096 517 / 60, 24 x 9 x 500 72 / 60, but
+// 24 x 9 x 128 23 / 25 in four shares; fp32 24 x 5 x 80 12.4 / 22.5, general fp32 4 layers x 9 x
+// 80 tokens x 1000 channels 14.5 / 26.4: not split. Of 760 sizes of each kind (1 to 48 layers of
+// 8 to 2048 channels, 80 to 1000 tokens) 6 to 16 take longer than unsplit now, by at most 18 to
+// 37 %, where a threshold of 80 tokens for all made it 78 to 244, up to 2.7 times.
+template <class C>
 int split_segments(const ScanParams &p) {
+    constexpr bool f32 = std::is_same<typename C::TIn, float>::value;
+    constexpr int64_t kPerChannels = C::MODE == kGeneral ? 40 : f32 ? 70 : 30, kPerCta = C::MODE == kPower && !f32 ? 5 : 15;
     const int64_t sms = device_sm_count();
-    // work items in chunks of 256 channels, tokens per chunk on average
-    const int64_t items = (static_cast<int64_t>(p.n_layers) * p.n_chunks * p.D + kMaxSlice - 1) / kMaxSlice;
-    const int64_t tokens = p.T_tot / p.n_chunks;
-    if (tokens < 80 || 2 * items > 3 * sms) return 1;
-    int segs = 8;
-    while (segs > 1 && (items * segs > 6 * sms || tokens < segs * 16)) segs /= 2;
-    return segs;
+    const int DS = pick_slice(p.D, C::MAXSLICE);
+    const int64_t pieces = static_cast<int64_t>(p.n_layers) * p.n_chunks;
+    const int64_t ctas = pieces * ((p.D + DS - 1) / DS), full = (pieces * p.D + kMaxSlice - 1) / kMaxSlice;
+    const int64_t tokens = p.T_tot / p.n_chunks;   // of a chunk on average: the offsets are on the device
+    if (tokens < 80 || 2 * full > 3 * sms) return 1;
+    for (int segs = 8; segs >= 4; segs /= 2)
+        if (full * segs <= 6 * sms && tokens >= segs * C::TILE && tokens * sms >= (kPerChannels * full + kPerCta * ctas) * segs)
+            return segs;
+    return 1;
 }
 
 // Two channels per thread, 128 registers, four CTAs of 256 channels per SM: power-form A with
@@ -1488,12 +1497,12 @@ cudaError_t launch_mode(const ScanParams &p, cudaStream_t stream) {
     const bool has_y = p.y != nullptr;
     const bool has_h0 = p.bank != nullptr;
     if (!has_y && !has_h0) {
-        const int segs = split_segments(p);
+        using Split = Cfg<TIn, false, false, MODE, 2, 16, 2, MODE == kGeneral ? 4 : 5, kTrajNone, kMaxSlice, 0, true>;
+        const int segs = split_segments<Split>(p);
         if (segs > 1) {
             ScanParams q = p;
             q.segments = segs;
-            return launch_cfg<Cfg<TIn, false, false, MODE, 2, 16, 2, MODE == kGeneral ? 4 : 5, kTrajNone, kMaxSlice, 0, true>>(
-                q, stream);
+            return launch_cfg<Split>(q, stream);
         }
     }
     if (has_y)

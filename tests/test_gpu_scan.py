@@ -577,10 +577,10 @@ def test_widths_that_slices_do_not_divide(cuda_device, D, kind, power):
 @pytest.mark.parametrize("kind", ["bf16", "f32"])
 @pytest.mark.parametrize("power", [True, False])
 @pytest.mark.parametrize("L,D,lens", [(1, 64, [4000]), (24, 256, [130]), (2, 1000, [0, 900, 17, 128, 129]),
-                                      (1, 8, [85]), (3, 512, [700, 1, 300, 160]), (2, 256, [97] * 70)])
+                                      (1, 8, [85]), (3, 512, [700, 1, 300, 160]), (2, 256, [97] * 20)])
 def test_split_chunks(cuda_device, kind, power, L, D, lens):
     """Captures with few work items share each chunk's tokens among a cluster's CTAs and
-    combine their states: 2, 4 and 8 shares, shares without tokens, chunks shorter than the
+    combine their states: 4 and 8 shares, shares without tokens, chunks shorter than the
     shares, a bad chunk beside good ones (skipped by its whole cluster), bf16 states, and
     the error against the oracle no larger than the one-CTA scan's tolerance."""
     import torch
@@ -658,3 +658,25 @@ def test_split_growing_modes(cuda_device, kind, power, T, first):
     tol = TOL_F32 if kind == "f32" else TOL_BF16
     err = np.abs(got - ref[0]).max(axis=0) / np.abs(ref[0]).max(axis=0)
     assert np.all(err < tol + nats * (T / 4 + 16 + 8) * 2.0 ** -24)
+
+
+@pytest.mark.parametrize("kind", ["bf16", "f32"])
+@pytest.mark.parametrize("L,D,n,T", [(24, 2048, 1, 80), (4, 1000, 9, 80), (24, 256, 9, 128), (24, 16, 60, 128)])
+def test_chunks_too_short_to_share(cuda_device, kind, L, D, n, T):
+    """Launches whose chunks are too short for the CTAs that sharing them would add (they took up to
+    2.7 times as long split) are not split: with a general A, whose token arithmetic is the same
+    in both launches, their states are those of the same chunks in a launch that fills the SMs,
+    bit for bit."""
+    import torch
+    dtype = torch.float32 if kind == "f32" else torch.bfloat16
+    gen = torch.Generator(device=cuda_device).manual_seed(D)
+    draw = lambda *shape: torch.randn(shape, generator=gen, device=cuda_device)
+    x, B = draw(L, n * T, D).to(dtype), (0.25 * draw(L, n * T, 16)).to(dtype)
+    dt = torch.nn.functional.softplus(draw(L, n * T, D) - 2).to(dtype)
+    A = -3 * torch.rand((L, D, 16), generator=gen, device=cuda_device)
+    off = lambda count: torch.arange(count + 1, device=cuda_device) * T
+    states, _ = _encode(cuda_device, x, dt, B, A, off(n))
+    r = 1 + 2 * 152 * 256 // (L * n * D)       # more than 1.5 CTAs of 256 channels per SM
+    many = [a.repeat(1, 1 + r, 1).contiguous() for a in (x, dt, B)]
+    full, _ = _encode(cuda_device, *many, A, off(n * (1 + r)))
+    assert torch.equal(states, full[:n])
