@@ -1262,15 +1262,25 @@ __global__ void __launch_bounds__(C::LB_THREADS, C::LB_BLOCKS)
 }
 
 // Channel slice of one CTA: the widest of 512 (if maxslice allows it), 256 and 128 channels that
-// divides the row; else the whole row if it fits, whatever its length, or slices of 256 whose
-// last one is narrower (its upper threads have no channels). Slices had to be a power of two
-// that divides D, so D = 1000 or 712 ran 125 or 89 CTAs of two threads per chunk: 2 layers x
-// 400 chunks x 200 tokens bf16, D = 1000: capture 3654 -> 225 us, readout 7035 -> 421 us,
-// general A (fp32) 2593 -> 540 us; D = 456: 1678 -> 128, 3219 -> 229, 1189 -> 275 us.
-int pick_slice(int D, int maxslice) {
+// divides the row; else the whole row if it fits, whatever its length, or the fewest slices of up
+// to 256, of equal width up to whole warps of two channels per thread (the last one is narrower:
+// its upper threads have no channels). Slices had to be a power of two that divides D, so D = 1000
+// or 712 ran 125 or 89 CTAs of two threads per chunk: 2 layers x 400 chunks x 200 tokens bf16,
+// D = 1000: capture 3654 -> 225 us, readout 7035 -> 421 us, general A (fp32) 2593 -> 540 us; D = 456:
+// 1678 -> 128, 3219 -> 229, 1189 -> 275 us. Equal slices against 256 and a rest: general fp32
+// readout of 2 layers x 138 x 687 tokens, D = 320, 298 us against 364. `narrow`: 64 channels.
+// For a general A or trajectories in launches that leave SMs idle, so that more SMs share the
+// exponentials or the stores (every 8th state of 1 x 40 x 200 tokens, general fp32, D = 320, 37 us,
+// equal slices 43; every state of 2 x 3 x 153, bf16 power form, D = 712, 39 us, 101), and for all
+// trajectories of a general A, whose deep ring leaves one fp32 CTA of 256 channels to an SM
+// (2 x 138 x 687, D = 448, 397 and 557).
+int pick_slice(int D, int maxslice, bool narrow) {
     for (int ds = kWideSlice; ds >= 128; ds /= 2)
         if (ds <= maxslice && D % ds == 0) return ds;
-    return D <= maxslice ? D : kMaxSlice;
+    if (D <= maxslice) return D;
+    if (narrow) return 64;
+    const int n = (D + kMaxSlice - 1) / kMaxSlice, width = (D + n - 1) / n;
+    return (width + 63) / 64 * 64;
 }
 
 // True when a full-width launch would have fewer CTAs than the device has SMs.
@@ -1296,7 +1306,8 @@ bool fits_quads(const ScanParams &p) {
 
 template <class C>
 cudaError_t launch_cfg(const ScanParams &p, cudaStream_t stream) {
-    const int DS = C::FIXDS ? C::FIXDS : pick_slice(p.D, C::MAXSLICE);
+    const bool idle = !C::SPLIT && (C::MODE == kGeneral || C::TRAJ != kTrajNone) && few_channels(p);
+    const int DS = C::FIXDS ? C::FIXDS : pick_slice(p.D, C::MAXSLICE, idle || (C::MODE == kGeneral && C::TRAJ != kTrajNone));
     if (DS % C::CPT != 0 || (C::FIXDS && p.D % DS != 0)) return cudaErrorInvalidValue;
     const int slices = (p.D + DS - 1) / DS;
     const StageLayout lay = stage_layout(C::TILE, DS, C::SZ, C::HAS_Y, C::CONV);
@@ -1370,7 +1381,7 @@ int split_segments(const ScanParams &p) {
     constexpr bool f32 = std::is_same<typename C::TIn, float>::value;
     constexpr int64_t kPerChannels = C::MODE == kGeneral ? 40 : f32 ? 70 : 30, kPerCta = C::MODE == kPower && !f32 ? 5 : 15;
     const int64_t sms = device_sm_count();
-    const int DS = pick_slice(p.D, C::MAXSLICE);
+    const int DS = pick_slice(p.D, C::MAXSLICE, false);
     const int64_t pieces = static_cast<int64_t>(p.n_layers) * p.n_chunks;
     const int64_t ctas = pieces * ((p.D + DS - 1) / DS), full = (pieces * p.D + kMaxSlice - 1) / kMaxSlice;
     const int64_t tokens = p.T_tot / p.n_chunks;   // of a chunk on average: the offsets are on the device
@@ -1427,7 +1438,7 @@ cudaError_t launch_t(const ScanParams &p, cudaStream_t stream) {
             // the corpus encode of 256- and 512-channel slices (the paper's layer width, the
             // ragged and wide workloads' slices) gets the slice fixed at compile time
             if constexpr (!HAS_H0) {
-                const int ds = pick_slice(p.D, kWideSlice);
+                const int ds = pick_slice(p.D, kWideSlice, false);
                 if (ds == 256 && p.D % 256 == 0)
                     return launch_cfg<Cfg<TIn, false, false, MODE, PRECOG_RESCALED_CPT, PRECOG_RESCALED_TILE,
                                           PRECOG_RESCALED_STAGES, PRECOG_RESCALED_MINB, kTrajNone, kWideSlice, 256>>(
@@ -1453,7 +1464,7 @@ cudaError_t launch_t(const ScanParams &p, cudaStream_t stream) {
                 return launch_pairs<TIn, HAS_Y, HAS_H0, kTrajNone>(p, stream);
             } else {
                 // 16-bit rows: 256- and 512-channel slices fixed at compile time
-                const int ds = pick_slice(p.D, kWideSlice);
+                const int ds = pick_slice(p.D, kWideSlice, false);
                 if (ds == 256 && p.D % 256 == 0)
                     return launch_cfg<Cfg<TIn, HAS_Y, HAS_H0, MODE, PRECOG_DIRECT_CPT, PRECOG_DIRECT_TILE,
                                           PRECOG_DIRECT_STAGES, PRECOG_DIRECT_MINB, kTrajNone, kWideSlice, 256>>(
@@ -1472,12 +1483,10 @@ cudaError_t launch_t(const ScanParams &p, cudaStream_t stream) {
             // 1000 chunks x 500 tokens fp32 1524 -> 1070 us, bf16 1096 -> 1032, with readout
             // 2126 -> 1419 and 1721 -> 1443. A readout launch that does not fill the SMs keeps
             // the deeper ring and the registers (24 x 3 x 500 bf16: 93 us, 102).
-            if constexpr (HAS_Y) {
-                if (few_channels(p))
-                    return p.D % 256 == 0
-                               ? launch_cfg<Cfg<TIn, HAS_Y, HAS_H0, MODE, 2, 16, 4, 3, kTrajNone, kMaxSlice, 256>>(p, stream)
-                               : launch_cfg<Cfg<TIn, HAS_Y, HAS_H0, MODE, 2, 16, 4, 3>>(p, stream);
-            }
+            if (few_channels(p))
+                return p.D % 256 == 0
+                           ? launch_cfg<Cfg<TIn, HAS_Y, HAS_H0, MODE, 2, 16, 4, 3, kTrajNone, kMaxSlice, 256>>(p, stream)
+                           : launch_cfg<Cfg<TIn, HAS_Y, HAS_H0, MODE, 2, 16, 4, 3>>(p, stream);
             if (p.D % 256 == 0)
                 return launch_cfg<Cfg<TIn, HAS_Y, HAS_H0, MODE, 2, 16, 2, 4, kTrajNone, kMaxSlice, 256>>(p, stream);
             return launch_cfg<Cfg<TIn, HAS_Y, HAS_H0, MODE, 2, 16, 2, 4>>(p, stream);

@@ -680,3 +680,47 @@ def test_chunks_too_short_to_share(cuda_device, kind, L, D, n, T):
     many = [a.repeat(1, 1 + r, 1).contiguous() for a in (x, dt, B)]
     full, _ = _encode(cuda_device, *many, A, off(n * (1 + r)))
     assert torch.equal(states, full[:n])
+
+
+@pytest.mark.parametrize("kind", ["bf16", "f32"])
+@pytest.mark.parametrize("power", [True, False])
+@pytest.mark.parametrize("D", [264, 320, 520])
+def test_equal_slices_in_launches_that_fill_the_sms(cuda_device, D, kind, power):
+    """Rows that 128 does not divide are cut into slices of equal width (264: 192 and 72, 520:
+    192, 192, 136), whose launches run more CTAs than SMs: capture, readout and trajectories
+    against the oracle. Where the power statement is false nothing of its slice is written:
+    with 320 channels of fp32 inputs those from 192 on."""
+    import torch
+    pg = _pg()
+    d = cuda_device
+    dtype = torch.float32 if kind == "f32" else torch.bfloat16
+    n, T = 220, 0
+    rng = np.random.default_rng(D)
+    lens = rng.integers(0, 24, size=n)
+    off = np.concatenate([[0], np.cumsum(lens)]).astype(np.int64)
+    T = int(off[-1])
+    x, dt, A, B, C = synth.host_scan_inputs(T, D, 16, seed=D)
+    if not power:
+        A = -rng.uniform(0.05, 3.0, size=(D, 16)).astype(np.float32)
+    a_kind = pg.PRECOG_A_POWER if power else pg.PRECOG_A_GENERAL
+    x, dt, B, C = (_t(a, d, dtype) for a in (x, dt, B, C))
+    offs = _t(off, d, torch.int64)
+    tol = TOL_F32 if kind == "f32" else TOL_BF16
+    states, y = _encode(d, x, dt, B, _t(A, d), offs, C=C, y_dtype=torch.float32, power=power)
+    capt, _ = _encode(d, x, dt, B, _t(A, d), offs, power=power)
+    ref_s, ref_y = oracle.scan(to_np(x), to_np(dt), A, to_np(B), off, C=to_np(C), want_y=True)
+    assert rel_err(to_np(y[0]), ref_y) < tol
+    assert rel_err(to_np(states[:, 0]), ref_s) < tol and rel_err(to_np(capt[:, 0]), ref_s) < tol
+    for stride in (3, 20):
+        ent = oracle.trajectory_offsets(off, stride)
+        traj = torch.full((int(ent[-1]), 1, D, 16), float("nan"), device=d)
+        pg.precog_encode_trajectory(pg.scan_inputs(x, dt, B, _t(A, d), a_kind=a_kind), offs, T, stride,
+                                    _t(ent, d, torch.int64), traj)
+        assert pg.precog_device_status()[0] == 0
+        assert rel_err(to_np(traj[:, 0]), oracle.trajectory(to_np(x), to_np(dt), A, to_np(B), off, stride)[0]) < tol
+    if power and kind == "f32" and D == 320:
+        A[200, 5] *= 1.5
+        out = torch.full_like(capt, 7.0)
+        pg.precog_encode_chunks(pg.scan_inputs(x, dt, B, _t(A, d), a_kind=a_kind), offs, T, out)
+        assert pg.precog_device_status()[1] == pg.PRECOG_DEV_BAD_A
+        assert (out[:, 0, 192:] == 7.0).all() and torch.equal(out[:, 0, :192], capt[:, 0, :192])
