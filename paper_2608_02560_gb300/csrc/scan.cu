@@ -1481,8 +1481,9 @@ cudaError_t launch_t(const ScanParams &p, cudaStream_t stream) {
             // stages and 128 registers let four CTAs share an SM's SFU (its bound: 16
             // exponentials per channel-token) where four stages left room for three: 4 layers x
             // 1000 chunks x 500 tokens fp32 1524 -> 1070 us, bf16 1096 -> 1032, with readout
-            // 2126 -> 1419 and 1721 -> 1443. A readout launch that does not fill the SMs keeps
-            // the deeper ring and the registers (24 x 3 x 500 bf16: 93 us, 102).
+            // 2126 -> 1419 and 1721 -> 1443. Launches that do not fill the SMs keep the deeper
+            // ring and the registers (bf16 readout 24 x 3 x 500: 93 us, 102; state-only prefill
+            // 24 x 1 x 500 x 64 channels: 59, 65; fp32 capture 24 x 7 x 79 x 64: 13.4, 14.4).
             if (few_channels(p))
                 return p.D % 256 == 0
                            ? launch_cfg<Cfg<TIn, HAS_Y, HAS_H0, MODE, 2, 16, 4, 3, kTrajNone, kMaxSlice, 256>>(p, stream)

@@ -724,3 +724,34 @@ def test_equal_slices_in_launches_that_fill_the_sms(cuda_device, D, kind, power)
         pg.precog_encode_chunks(pg.scan_inputs(x, dt, B, _t(A, d), a_kind=a_kind), offs, T, out)
         assert pg.precog_device_status()[1] == pg.PRECOG_DEV_BAD_A
         assert (out[:, 0, 192:] == 7.0).all() and torch.equal(out[:, 0, :192], capt[:, 0, :192])
+
+
+@pytest.mark.parametrize("kind", ["bf16", "f32"])
+@pytest.mark.parametrize("D", [64, 256, 512])
+def test_general_launches_of_few_channels(cuda_device, D, kind):
+    """Captures and state-only prefills with a general A that leave SMs idle take the readout's
+    deeper ring (four stages): chunks of no, one, few and many tiles."""
+    import torch
+    pg = _pg()
+    dtype = torch.float32 if kind == "f32" else torch.bfloat16
+    lens = [0, 1, 16, 65, 79, 80, 130]           # 53 tokens on average: not shared
+    off = np.concatenate([[0], np.cumsum(lens)]).astype(np.int64)
+    x, dt, _, B, _ = synth.host_scan_inputs(int(off[-1]), D, 16, seed=D)
+    rng = np.random.default_rng(D)
+    A = -rng.uniform(0.05, 3.0, size=(D, 16)).astype(np.float32)
+    x, dt, B = (_t(a, cuda_device, dtype) for a in (x, dt, B))
+    tol = TOL_F32 if kind == "f32" else TOL_BF16
+    capt, _ = _encode(cuda_device, x, dt, B, _t(A, cuda_device), _t(off, cuda_device, torch.int64))
+    ref, _ = oracle.scan(to_np(x), to_np(dt), A, to_np(B), off)
+    assert rel_err(to_np(capt[:, 0]), ref) < tol
+    n, t = 3, 100
+    bank = rng.standard_normal((2, 1, D, 16)).astype(np.float32)
+    h = torch.full((n, 1, D, 16), float("nan"), device=cuda_device)
+    pg.precog_prefill_from_state(pg.scan_inputs(x[:n * t], dt[:n * t], B[:n * t], _t(A, cuda_device)), n, t,
+                                 _t(bank, cuda_device), torch.tensor([1, -1, 0], device=cuda_device), state_out=h)
+    assert pg.precog_device_status()[0] == 0
+    for q, row in enumerate([1, -1, 0]):
+        sl = slice(q * t, (q + 1) * t)
+        ref, _ = oracle.rollout(to_np(x[sl]), to_np(dt[sl]), A, to_np(B[sl]),
+                                h0=bank[row, 0] if row >= 0 else np.zeros((D, 16)))
+        assert rel_err(to_np(h[q, 0]), ref) < tol
