@@ -86,7 +86,8 @@ enum Mode { kGeneral = 0, kPower = 1 };
 constexpr int kTrajNone = 0, kTrajDirect = 1, kTrajRescaled = 2;
 
 template <typename TIn_, bool HAS_Y_, bool HAS_H0_, int MODE_, int CPT_, int TILE_, int STAGES_,
-          int MINB_, int TRAJ_ = kTrajNone, int MAXSLICE_ = kMaxSlice, int FIXDS_ = 0, bool SPLIT_ = false>
+          int MINB_, int TRAJ_ = kTrajNone, int MAXSLICE_ = kMaxSlice, int FIXDS_ = 0, bool SPLIT_ = false,
+          bool PAIRS_ = false>
 struct Cfg {
     using TIn = TIn_;
     // Channel slice known at compile time (0: a launch argument). A constant slice turns
@@ -94,9 +95,11 @@ struct Cfg {
     static constexpr int FIXDS = FIXDS_;
     // A cluster of CTAs per work item, each with a share of the chunk's tokens (see combine).
     static constexpr bool SPLIT = SPLIT_;
+    // The shape of launch_pairs: two channels per thread where other inputs take four.
+    static constexpr bool PAIRS = PAIRS_;
     // 256-channel slices that stand in for 512-channel ones: the power statement is verified
     // for the 512 channels together, as by those.
-    static constexpr bool WIDE_CHECK = MODE_ == kPower && CPT_ == 2 && (SPLIT_ || TRAJ_ != kTrajNone || MINB_ == 4);
+    static constexpr bool WIDE_CHECK = MODE_ == kPower && CPT_ == 2 && (SPLIT_ || PAIRS_ || TRAJ_ != kTrajNone);
     // Widest channel slice of one CTA. Each CTA stages its slice of every token row; a
     // slice narrower than the row turns the row into separate pieces, and HBM serves
     // short scattered pieces far below its streaming rate, so rows up to 512 channels
@@ -111,7 +114,7 @@ struct Cfg {
     static constexpr int TRAJ = TRAJ_;
     static constexpr int MODE = MODE_, CPT = CPT_, TILE = TILE_, STAGES = STAGES_;
     // trajectory states leave through shared memory (see store_trajectory)
-    static constexpr bool STAGED = TRAJ_ != kTrajNone && MODE_ == kPower && CPT_ == 2 && MINB_ == 4;
+    static constexpr bool STAGED = TRAJ_ != kTrajNone && PAIRS_;
     static constexpr bool CONV = !std::is_same<TIn_, float>::value;
     static constexpr int SZ = sizeof(TIn_);
     static constexpr bool RESCALED = MODE_ == kPower && !HAS_Y_ && TRAJ_ != kTrajDirect;
@@ -163,21 +166,11 @@ __host__ __device__ inline StageLayout stage_layout(int tile, int DS, int sz, bo
 template <typename TIn, int CPT>
 __device__ __forceinline__ void load_chan(const unsigned char *p, float (&v)[CPT], uint32_t &neg) {
     if constexpr (std::is_same<TIn, float>::value) {
-        if constexpr (CPT == 2) {
-            const float2 q = *reinterpret_cast<const float2 *>(p);
-            v[0] = q.x;
-            v[1] = q.y;
-        } else {
-            const float4 q = *reinterpret_cast<const float4 *>(p);
-            v[0] = q.x;
-            v[1] = q.y;
-            v[2] = q.z;
-            v[3] = q.w;
-        }
-        uint32_t s = 0;
-#pragma unroll
-        for (int j = 0; j < CPT; ++j) s |= __float_as_uint(v[j]);
-        neg = s & 0x80000000u;
+        static_assert(CPT == 2, "fp32 inputs: two channels per thread");
+        const float2 q = *reinterpret_cast<const float2 *>(p);
+        v[0] = q.x;
+        v[1] = q.y;
+        neg = (__float_as_uint(q.x) | __float_as_uint(q.y)) & 0x80000000u;
     } else {
         uint32_t w[CPT / 2];
         if constexpr (CPT == 2) {
@@ -1401,8 +1394,8 @@ int split_segments(const ScanParams &p) {
 template <typename TIn, bool HAS_Y, bool HAS_H0, int TRAJ>
 cudaError_t launch_pairs(const ScanParams &p, cudaStream_t stream) {
     if (p.D % kMaxSlice == 0)
-        return launch_cfg<Cfg<TIn, HAS_Y, HAS_H0, kPower, 2, 16, 2, 4, TRAJ, kMaxSlice, kMaxSlice>>(p, stream);
-    return launch_cfg<Cfg<TIn, HAS_Y, HAS_H0, kPower, 2, 16, 2, 4, TRAJ, kMaxSlice>>(p, stream);
+        return launch_cfg<Cfg<TIn, HAS_Y, HAS_H0, kPower, 2, 16, 2, 4, TRAJ, kMaxSlice, kMaxSlice, false, true>>(p, stream);
+    return launch_cfg<Cfg<TIn, HAS_Y, HAS_H0, kPower, 2, 16, 2, 4, TRAJ, kMaxSlice, 0, false, true>>(p, stream);
 }
 
 // Shapes: the rescaled capture kernel (the corpus-encode hot loop) and the
