@@ -133,6 +133,10 @@ typedef struct precog_scan_inputs {
  *               non-decreasing with d_offsets[n_chunks] <= T_tot (checked on
  *               the device: a bad chunk is skipped and flags
  *               PRECOG_DEV_BAD_OFFSETS). A zero-length chunk captures zeros.
+ *   T_tot       token rows of x, dt, B and C per layer. The rows of d_offsets are on
+ *               the device, so the launch is shaped by T_tot / n_chunks: a T_tot far
+ *               beyond what d_offsets covers costs time (a few microseconds), never
+ *               correctness.
  *   states_out  device [n_chunks][L_total][D][N] in state_dtype (F32 or BF16,
  *               rounded to nearest even once, at capture); the call writes
  *               layers layer0 .. layer0+L-1 and nothing else. May be NULL
@@ -140,6 +144,10 @@ typedef struct precog_scan_inputs {
  *   y_out       device [L][T_tot][D] in y_dtype (F32 or BF16): readout after
  *               every token (used to check Theorem 1), or NULL for capture
  *               only. Rows outside every chunk are left untouched.
+ * Without y_out, a call with few (layer, chunk) pairs shares each chunk's tokens among
+ * several CTAs and combines their partial states, so the last bits of a state may
+ * depend on n_layers, n_chunks, D and T_tot of the call (both forms agree with the
+ * recurrence within the same tolerance); calls of the same shape repeat bit for bit.
  * Returns PRECOG_OK once the work is enqueued.
  */
 precog_status precog_encode_chunks(const precog_scan_inputs *in, const int64_t *d_offsets,
@@ -173,7 +181,7 @@ precog_status precog_encode_chunks_ordered(const precog_scan_inputs *in, const i
  * precog_encode_chunks and keep the state after every `stride`-th token and
  * after the chunk's last token. Chunk c keeps K_c = ceil(len_c / stride)
  * states (K = N_c / k in the paper; stride 1 keeps every state, stride >=
- * len_c keeps only the final, PRECOG state). Uses the direct update.
+ * len_c keeps only the final, PRECOG state).
  *   d_entry_offsets  device int64 [n_chunks+1]: prefix sums of K_c; a chunk
  *                    whose count disagrees with its length is skipped and
  *                    flags PRECOG_DEV_BAD_OFFSETS
@@ -194,9 +202,11 @@ precog_status precog_encode_trajectory(const precog_scan_inputs *in, const int64
  * row i* of the key index with the highest dot product <query_q, key_i>
  * (unit-norm keys and queries make this the cosine similarity of the paper).
  * Exact top-1, not an approximate index. Scores accumulate in fp32 from the
- * stored values; ties go to the lowest row; a NaN score never wins; if no row
- * has a comparable score (M == 0, or every score NaN) the result is index -1 and
- * score NaN, and the call still returns PRECOG_OK.
+ * stored values (F32 indexes: in an order that depends on dim alone, so that a row
+ * scores the same bits alone or in a batch, as top-1 or in a top-k call); ties go to
+ * the lowest row; a NaN score never wins; if no row has a comparable score (M == 0,
+ * or every score NaN) the result is index -1 and score NaN, and the call still
+ * returns PRECOG_OK.
  *
  *   index          device [M][dim] keys in index_dtype (F16, BF16 or F32)
  *   queries        device [n_queries][dim], same dtype as the index

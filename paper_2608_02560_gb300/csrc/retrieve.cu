@@ -364,7 +364,7 @@ __global__ void finalize_topk_kernel(const unsigned long long *__restrict__ part
 // lanes by halving exchanges (each step sends the half of the sums that the other lane
 // keeps): 16 exchanges for 16 sums where separate butterflies take 80, in the same tree for
 // every row, so equal rows score equally. Bound: HBM up to about 8 queries, then the FMA
-// pipe (56 % busy: three warps per scheduler, exchanges and key updates between the sums).
+// pipe (59 % busy: three warps per scheduler, exchanges and key updates between the sums).
 // Top-1 / top-3, us, before (a pass per 4 queries / per query) -> now:
 //   8 queries, 50,021 x 384      53 / 170 ->  24 /  24   (77 MB: 11 us)
 //   23                          144 / 449 ->  38 /  42

@@ -1289,7 +1289,7 @@ bool few_channels(const ScanParams &p) {
 }
 
 // Whether six CTAs per SM of four channels per thread take a launch in fewer rounds (counted in
-// CTAs per SM) than four of two channels per thread, whose tokens cost 7 % more.
+// CTAs per SM) than four of two channels per thread, whose tokens cost 7 % more (16-bit inputs).
 bool fits_quads(const ScanParams &p) {
     const int64_t items = (static_cast<int64_t>(p.n_layers) * p.n_chunks * p.D + kMaxSlice - 1) / kMaxSlice;
     const int64_t sms = device_sm_count();
@@ -1385,12 +1385,13 @@ int split_segments(const ScanParams &p) {
     return 1;
 }
 
-// Two channels per thread, 128 registers, four CTAs of 256 channels per SM: power-form A with
-// fp32 inputs. Their tiles are twice as large, so that with four channels per thread three CTAs
-// of two warps were left to an SM; this shape has 16 warps: 1 layer x 500 chunks x 1000 tokens
+// Two channels per thread: power-form A with fp32 inputs, and trajectories that fill the SMs. The
+// ring of 256 fp32 channels takes 68 KB, so three CTAs share an SM whatever their registers, and
+// with two channels per thread they are 12 warps instead of 6: 1 layer x 500 chunks x 1000 tokens
 // capture 274 -> 231 us, 1 x 100 x 300 x 2048 144 -> 112; readout 24 x 30 x 500 370 -> 290,
-// 1 x 100 x 300 x 2048 276 -> 215. (bf16 captures of this shape take 215 -> 234 us, readouts
-// 190 -> 209.)
+// 1 x 100 x 300 x 2048 276 -> 215. The buffers of staged trajectories leave two CTAs of fp32 inputs
+// and four of bf16 ones (16 warps, 122 registers). bf16 captures and readouts keep four channels per
+// thread (in this shape 215 -> 234 us and 190 -> 209).
 template <typename TIn, bool HAS_Y, bool HAS_H0, int TRAJ>
 cudaError_t launch_pairs(const ScanParams &p, cudaStream_t stream) {
     if (p.D % kMaxSlice == 0)
@@ -1470,13 +1471,14 @@ cudaError_t launch_t(const ScanParams &p, cudaStream_t stream) {
                                       PRECOG_DIRECT_STAGES, PRECOG_DIRECT_MINB, kTrajNone, kWideSlice>>(p, stream);
             }
         } else {
-            // general A keeps 16 exponent coefficients per channel: 2 channels per thread. Two
-            // stages and 128 registers let four CTAs share an SM's SFU (its bound: 16
-            // exponentials per channel-token) where four stages left room for three: 4 layers x
-            // 1000 chunks x 500 tokens fp32 1524 -> 1070 us, bf16 1096 -> 1032, with readout
-            // 2126 -> 1419 and 1721 -> 1443. Launches that do not fill the SMs keep the deeper
-            // ring and the registers (bf16 readout 24 x 3 x 500: 93 us, 102; state-only prefill
-            // 24 x 1 x 500 x 64 channels: 59, 65; fp32 capture 24 x 7 x 79 x 64: 13.4, 14.4).
+            // general A keeps 16 exponent coefficients per channel: 2 channels per thread. The
+            // more CTAs share an SM's SFU (the bound: 16 exponentials per channel-token) the better:
+            // with two stages and 128 registers four of bf16 inputs and three of fp32 ones (68 KB
+            // rings), with four stages three (readouts two) and one. 4 layers x 1000 chunks x 500
+            // tokens fp32 1524 -> 1070 us, bf16 1096 -> 1032, with readout 2126 -> 1419 and 1721 ->
+            // 1443. Launches that do not fill the SMs keep the deeper ring and the registers (bf16
+            // readout 24 x 3 x 500: 93 us, 102; state-only prefill 24 x 1 x 500 x 64 channels: 59, 65;
+            // fp32 capture 24 x 7 x 79 x 64: 13.4, 14.4).
             if (few_channels(p))
                 return p.D % 256 == 0
                            ? launch_cfg<Cfg<TIn, HAS_Y, HAS_H0, MODE, 2, 16, 4, 3, kTrajNone, kMaxSlice, 256>>(p, stream)

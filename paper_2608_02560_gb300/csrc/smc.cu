@@ -391,8 +391,9 @@ __global__ void __launch_bounds__(kSlotThreads)
 // private ring of 16-byte asynchronous copies in shared memory: no barrier, no producer
 // and no wait on another thread. (One producer thread queueing a bulk copy per deposit
 // cost about 250 ns per deposit and CTA, whatever the size: 1.0 TB/s on 2 KB ranges.)
-// kRingChunks chunks per thread are in flight: 18 deposits of a tile of up to 4 KB, 9 of
-// 8 KB, 4 of 16 KB, 3 of 24 KB, 72 KB per CTA and two CTAs per SM. Narrower or wider tiles
+// The ring holds kRingChunks chunks per thread, 72 KB per CTA and two CTAs per SM, and all of its
+// groups but the one being folded are in flight: 17 deposits of a tile of up to 4 KB (34 of 2 KB
+// and 68 of 1 KB, side by side), 8 of 8 KB, 3 of 16 KB, 2 of 24 KB. Narrower or wider tiles
 // and shorter or longer rings were slower (4096 states below: 16 KB tiles 147 us; a ring of
 // 12 chunks 158 us; 24 chunks the same as 18 and 66 against 64 us in the second case).
 //
@@ -702,11 +703,11 @@ cudaError_t launch_smc_consolidate(float *sem, int64_t n_slots, int64_t elems, c
     const int64_t blocks = (elems / vec + kConsThreads - 1) / kConsThreads;
     if (blocks > 0x7fffffffLL) return cudaErrorInvalidConfiguration;
     const unsigned grid = static_cast<unsigned>(blocks);
-    // Few slots: CTAs over pieces of (slot, element range). Each piece (each tile beyond
-    // kWindow deposits) reads all n slot ids from L2: n_slots / 2048 of its state bytes
-    // with 16 KB ranges, so it pays up to 256 slots. Rows of whole 16-byte chunks stream
-    // through the copy ring; other rows take the register per-slot kernel (whose
-    // 2048-element ranges read n_slots / 512).
+    // Few slots: CTAs over pieces of (slot, element range). Rows of whole 16-byte chunks stream
+    // through the copy rings: a CTA reads all n slot ids from L2 to count the deposits of up to
+    // kTallySlots slots, one per thread, and again for each piece (each tile beyond kWindow
+    // deposits) to list its slot's. Other rows take the register per-slot kernel, whose CTAs
+    // of 2048 elements read n_slots / 512 of their state bytes in slot ids.
     const int64_t size = states_dtype == PRECOG_BF16 ? 2 : 4;
     const int64_t units = (elems * size + kUnitBytes - 1) / kUnitBytes;
     if (n_slots >= 1 && n_slots <= kTallySlots && elems * size % 16 == 0 && units < 0x7fffffffLL) {

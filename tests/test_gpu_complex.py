@@ -297,7 +297,7 @@ def test_complex_rescaled_capture_regimes(cuda_device, form, regime):
                                     (256, [137] * 70)])
 def test_complex_split_chunks(cuda_device, D, lens, form, in16):
     """Captures with few work items share each chunk's tokens among a cluster's CTAs and
-    combine their states: 2, 4 and 8 shares, shares without tokens, chunks shorter than the
+    combine their states: 4 and 8 shares, shares without tokens, chunks shorter than the
     shares, bf16 states. Slow decays (small dt in the second half) keep the early segments'
     states and their many turns of phase in the result, and with them the per-token rounding
     of every form (1e-5 and more over 2500 tokens), so the bound is the unsplit scan's own
