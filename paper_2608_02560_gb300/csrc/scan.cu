@@ -95,9 +95,8 @@ struct Cfg {
     static constexpr int FIXDS = FIXDS_;
     // A cluster of CTAs per work item, each with a share of the chunk's tokens (see combine).
     static constexpr bool SPLIT = SPLIT_;
-    // The shape of launch_pairs: two channels per thread where other inputs take four.
-    static constexpr bool PAIRS = PAIRS_;
-    // 256-channel slices that stand in for 512-channel ones: the power statement is verified
+    // 256-channel slices that stand in for 512-channel ones (PAIRS_: the shape of launch_pairs,
+    // two channels per thread where other inputs take four): the power statement is verified
     // for the 512 channels together, as by those.
     static constexpr bool WIDE_CHECK = MODE_ == kPower && CPT_ == 2 && (SPLIT_ || PAIRS_ || TRAJ_ != kTrajNone);
     // Widest channel slice of one CTA. Each CTA stages its slice of every token row; a
