@@ -1287,13 +1287,23 @@ bool few_channels(const ScanParams &p) {
     return static_cast<int64_t>(p.n_layers) * p.n_chunks * p.D < static_cast<int64_t>(device_sm_count()) * kMaxSlice;
 }
 
-// Whether six CTAs per SM of four channels per thread take a launch in fewer rounds (counted in
-// CTAs per SM) than four of two channels per thread, whose tokens cost 7 % more (16-bit inputs).
+// Whether trajectories with the rescaled update (16-bit inputs) go four channels per thread and
+// store plainly, in the captures' shape, or two and staged (launch_pairs), whose tokens cost 5 %
+// more. Plain stores pay from strides of 64 with bf16 states and 128 (100 in slices of other than
+// 256 channels) with fp32 ones. A CTA of 256 channels is two warps in the first
+// shape: an odd number of them per SM leaves two of its four schedulers a warp behind, while
+// the second's four warps load all alike; in CTAs of one warp (rows that 128 divides but not
+// 256) it is the last round that counts. us, every 250th fp32 state, 152 n CTAs of 256 channels,
+// first / second shape: n = 6 (700 tokens) 234 / 245, 7 301 / 281, 12 438 / 462, 20 (420 tokens)
+// 435 / 460, 27 (311) 454 / 462; stride 64, n = 8 (600) 297 / 282, bf16 270 / 278. Second / first of
+// D = 128: n = 7 0.97, 11 1.02, 21 1.06; D = 64: 0.61; 192: 0.92; 320: 1.03.
 bool fits_quads(const ScanParams &p) {
+    if (p.D < 256 && p.D % 128 != 0) return false;   // dead lanes
+    const int ds = pick_slice(p.D, kWideSlice, false);
+    if (p.traj_stride < (p.traj_dtype != PRECOG_F32 ? 64 : ds == 256 ? 128 : 100)) return false;
     const int64_t items = (static_cast<int64_t>(p.n_layers) * p.n_chunks * p.D + kMaxSlice - 1) / kMaxSlice;
-    const int64_t sms = device_sm_count();
-    const int64_t quads = (items + 6 * sms - 1) / (6 * sms) * 6, pairs = (items + 4 * sms - 1) / (4 * sms) * 4;
-    return 100 * quads <= 107 * pairs;
+    const int64_t per_sm = (items + device_sm_count() - 1) / device_sm_count();
+    return ds % 256 == 0 ? per_sm > 2 && 200 * ((per_sm + 1) / 2) <= 105 * per_sm : per_sm > 8;
 }
 
 template <class C>
@@ -1403,13 +1413,11 @@ cudaError_t launch_pairs(const ScanParams &p, cudaStream_t stream) {
 template <typename TIn, bool HAS_Y, bool HAS_H0, int MODE, int TRAJ = kTrajNone>
 cudaError_t launch_t(const ScanParams &p, cudaStream_t stream) {
     if constexpr (TRAJ != kTrajNone) {
-        // power form: the rescaled or (short strides) the direct update, in the fp32 shape for
-        // any input but for wide strides of 16-bit chunks that fill rounds of the captures' shape
-        // (in that shape and in the fp32 one, us: stride 216, 4 x 208 x 2611 tokens 837, 882;
-        // stride 1000, 4 x 1000 x 750 1076, 1088; stride 100, 4 x 250 x 750 374, 345)
+        // power form: the rescaled or (short strides) the direct update, in the fp32 shape but
+        // for wide strides of 16-bit inputs where the captures' shape is faster (fits_quads)
         if constexpr (MODE == kPower) {
             if constexpr (TRAJ == kTrajRescaled && !std::is_same<TIn, float>::value)
-                if (p.traj_stride >= 64 && fits_quads(p))
+                if (fits_quads(p))
                     return p.D % 256 == 0 && p.D % 512 != 0
                                ? launch_cfg<Cfg<TIn, false, false, kPower, PRECOG_RESCALED_CPT, PRECOG_RESCALED_TILE,
                                                 PRECOG_RESCALED_STAGES, PRECOG_RESCALED_MINB, TRAJ, kWideSlice, 256>>(p, stream)
